@@ -1685,39 +1685,50 @@ __global__ void __launch_bounds__(512, MINB) bpsf_persistent(const __grid_consta
     bool waiting = false;
     unsigned long long wait_start = 0;
     for (;;) {
-        if (tid == 0) {
-            int pick = -1;
-            bool all_done = true;
-            const int ns = kp.n_streams;
-            const int start = (cur >= 0) ? cur : (int)(blockIdx.x % (unsigned)ns);
-            for (int k = 0; k < ns; ++k) {
-                const int sid = (start + k) % ns;
-                const StreamDev &sd = kp.streams[sid];
+        if (warp == 0) {
+            // Lane k looks at stream k, so the streams' counters are read in one
+            // round trip.  A block stays with its stream while there is work to
+            // claim there; when it has to move, the blocks spread over the streams
+            // that still have work (block b takes the (b mod n)-th of the n).
+            // Taking the next one in order instead sent the blocks of a finished
+            // job to one shard of the next job, whose counters they then queued on:
+            // four [[144]] jobs (p = 0.02 .. 0.08, 250 000 shots each) in one launch
+            // took 135.6 ms that way, and the four one after another 101 ms.
+            bool claimable = false, done = true;
+            if (lane < kp.n_streams) {
+                const StreamDev &sd = kp.streams[lane];
                 const StreamCounters *c = sd.ctr;
                 if (sd.flags & kServe) {
                     const long long pub = ld_acquire_sys_s64(sd.serve.published);
                     const long long sn = (long long)ld_vol_u64(&c->shot_next);
                     const unsigned long long ttot = ld_vol_u64(&c->rec_count) * (unsigned long long)sd.code.n_trials;
-                    const bool claimable = sn < pub || ld_vol_u64(&c->ticket_next) < ttot;
-                    if (claimable && pick < 0) pick = sid;
-                    if (claimable || !*sd.serve.stop) all_done = false;
-                    continue;
+                    claimable = sn < pub || ld_vol_u64(&c->ticket_next) < ttot;
+                    done = !claimable && *sd.serve.stop;
+                } else {
+                    const unsigned long long n = (unsigned long long)sd.job.n_shots;
+                    const unsigned long long shot_next = ld_vol_u64(&c->shot_next);
+                    const unsigned long long init_done = ld_vol_u64(&c->init_done);
+                    __threadfence();
+                    const unsigned long long rc = ld_vol_u64(&c->rec_count);
+                    const unsigned long long tk = ld_vol_u64(&c->ticket_next);
+                    const bool trials = sd.code.w > 0 && !(sd.flags & kNoTickets);
+                    const unsigned long long ttot = trials ? rc * (unsigned long long)sd.code.n_trials : 0ull;
+                    claimable = shot_next < n || tk < ttot;
+                    done = shot_next >= n && init_done >= n && tk >= ttot;
                 }
-                const unsigned long long n = (unsigned long long)sd.job.n_shots;
-                const unsigned long long shot_next = ld_vol_u64(&c->shot_next);
-                const unsigned long long init_done = ld_vol_u64(&c->init_done);
-                __threadfence();
-                const unsigned long long rc = ld_vol_u64(&c->rec_count);
-                const unsigned long long tk = ld_vol_u64(&c->ticket_next);
-                const bool trials = sd.code.w > 0 && !(sd.flags & kNoTickets);
-                const unsigned long long ttot = trials ? rc * (unsigned long long)sd.code.n_trials : 0ull;
-                const bool claimable = shot_next < n || tk < ttot;
-                const bool done = shot_next >= n && init_done >= n && tk >= ttot;
-                if (claimable && pick < 0) pick = sid;
-                if (!done) all_done = false;
             }
-            hdr->stream = pick;
-            hdr->cmd = pick >= 0 ? 1 : (all_done ? 2 : 0);
+            const unsigned cm = __ballot_sync(FULLMASK, claimable);
+            const bool all_done = __all_sync(FULLMASK, done);
+            if (lane == 0) {
+                int pick = -1;
+                if (cur >= 0 && ((cm >> cur) & 1u)) {
+                    pick = cur;
+                } else if (cm) {
+                    pick = (int)__fns(cm, 0u, (int)(blockIdx.x % (unsigned)__popc(cm)) + 1);
+                }
+                hdr->stream = pick;
+                hdr->cmd = pick >= 0 ? 1 : (all_done ? 2 : 0);
+            }
         }
         __syncthreads();
         const int cmd = hdr->cmd, sid = hdr->stream;
