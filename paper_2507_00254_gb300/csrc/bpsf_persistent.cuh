@@ -161,17 +161,72 @@ template <int FB> __device__ __forceinline__ unsigned flip_count(unsigned f) { r
 template <int FB> __device__ __forceinline__ unsigned flip_bump(unsigned f) { return (f ^ (1u << (8 * FB - 1))) + 1u; }
 
 // ---------------------------------------------------------------------------
-// C phase: check-node update, Eq. (c2v).  For row j with V2C inputs q_k:
-//   neg = s_j xor (xor_k [q_k < 0]),  m1 = min |q_k| (first argmin k1),
-//   m2 = min over k != k1,  r_k = (neg xor [q_k < 0]) ? -a : a,
-//   a = alpha * (k == k1 ? m2 : m1),
-// which equals the explicit "min and sign product over the other variables"
-// bit for bit (min is exact; the sign factors are exact), independently of
-// the order the row's edges are stored in.  V2C messages are never -0 (each
-// is a fold that starts at a channel LLR > 0, and an exact cancellation
-// rounds to +0), so the sign bit of q_k is [q_k < 0] and the sign product is
-// an XOR of sign bits.  m2 = min(m2, max(m1, a)) keeps the second smallest
-// value branch-free, equal to m1 on ties.
+// Arithmetic of the phases.  A lane serves V adjacent slots (1, 2 or 4); two
+// slots' values share one packed FP32 operation, each half rounded on its own.
+// ---------------------------------------------------------------------------
+template <int V> struct VecF;
+template <> struct VecF<1> { typedef float T; };
+template <> struct VecF<2> { typedef float2 T; };
+template <> struct VecF<4> { typedef float4 T; };
+
+template <int V>
+__device__ __forceinline__ void vload(float (&x)[V], const typename VecF<V>::T *p) {
+    const typename VecF<V>::T t = *p;
+#pragma unroll
+    for (int c = 0; c < V; ++c) x[c] = reinterpret_cast<const float *>(&t)[c];
+}
+template <int V>
+__device__ __forceinline__ void vstore(typename VecF<V>::T *p, const float (&x)[V]) {
+    typename VecF<V>::T t;
+#pragma unroll
+    for (int c = 0; c < V; ++c) reinterpret_cast<float *>(&t)[c] = x[c];
+    *p = t;
+}
+
+// o = a * b, a + b, a - b, slot by slot.
+#define BPSF_VOP(name, op, scalar)                                                                                  \
+    template <int V>                                                                                                \
+    __device__ __forceinline__ void name(float (&o)[V], const float (&a)[V], const float (&b)[V]) {                 \
+        if (V == 1) {                                                                                               \
+            o[0] = scalar(a[0], b[0]);                                                                              \
+        } else {                                                                                                    \
+            _Pragma("unroll") for (int c = 0; c + 1 < V; c += 2)                                                    \
+                asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t" op                     \
+                    " x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"                                                         \
+                    : "=f"(o[c]), "=f"(o[c + 1])                                                                    \
+                    : "f"(a[c]), "f"(a[c + 1]), "f"(b[c]), "f"(b[c + 1]));                                          \
+        }                                                                                                           \
+    }
+BPSF_VOP(vmul, "mul.rn.f32x2", __fmul_rn)
+BPSF_VOP(vadd, "add.rn.f32x2", __fadd_rn)
+BPSF_VOP(vsub, "sub.rn.f32x2", __fsub_rn)
+#undef BPSF_VOP
+
+// min(|a|, |b|) with the product of the two signs: one instruction.
+__device__ __forceinline__ float min_sign(float a, float b) {
+    float o;
+    asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(o) : "f"(a), "f"(b));
+    return o;
+}
+template <int V>
+__device__ __forceinline__ void vmins(float (&o)[V], const float (&a)[V], const float (&b)[V]) {
+#pragma unroll
+    for (int c = 0; c < V; ++c) o[c] = min_sign(a[c], b[c]);
+}
+
+// ---------------------------------------------------------------------------
+// Check-node update, Eq. (c2v): with a o b = (the signs' product) min(|a|, |b|),
+//   out_k = seed o (o over k' != k of alpha q_k'),
+// seed = 2^100 with the sign of the row's syndrome bit.  The minimum is exact
+// and multiplication by alpha > 0 is monotone, so this equals alpha times the
+// minimum over the other variables, clamped at 2^100, bit for bit and in any
+// grouping; the sign is the XOR of the sign bits (V2C messages are never -0:
+// each is a fold that starts at a channel LLR > 0, and an exact cancellation
+// rounds to +0).
+//
+// A six-wide row takes 14 operations o for its outputs.  Keeping the two
+// smallest magnitudes and selecting per output took seven ALU operations per
+// edge, and the loop ran at 75 % of the ALU pipe.
 // ---------------------------------------------------------------------------
 // C2V magnitudes are clamped here (2^100): never reached with a fixed alpha at
 // the configurations; keeps messages finite when adaptive damping tends to 1.
@@ -189,90 +244,84 @@ __device__ __forceinline__ float damping(const CodeDev &cd, int t) {
     return cd.alpha > 0.f ? cd.alpha : __fsub_rn(1.0f, tiny);
 }
 
-template <int DC, bool REG>
-struct CTask {
-    float v[DC];
-    float *p;       // message of edge rank 0 of this (row, slot); rank k sits k*M*S further
-    unsigned sall;  // bit 31: s_j xor the sign bits of all inputs
-    int deg;
-    bool on;
-};
+// Seeds of a row for V slots: syndrome bits in the low bits of sb.  NEG: the
+// outputs carry the opposite sign (see the V phase).
+template <int V, bool NEG>
+__device__ __forceinline__ void row_seed(float (&sd)[V], unsigned sb) {
+#pragma unroll
+    for (int c = 0; c < V; ++c)
+        sd[c] = __uint_as_float((((NEG ? ~sb : sb) << (31 - c)) & 0x80000000u) | 0x71800000u);
+}
 
-// Task tau = j*S + s of the interleaved team layout: row j of slot s.
-template <int DC, bool REG>
-__device__ __forceinline__ void c_load(CTask<DC, REG> &t, const LayoutMem &L, const TeamMem &T, int MS, int lgS,
-                                       int tau, bool on) {
-    t.on = on;
-    if (!on) return;
-    t.deg = REG ? DC : (int)L.row_deg[tau >> lgS];
-    t.p = T.m + tau;
-    t.sall = (T.syn[tau >> 5] >> (tau & 31)) << 31;
+// x_k (already times alpha) -> out_k, in place; edges a row does not have hold
+// +infinity (neutral).  Pairs' products, a prefix and a suffix scan over the
+// pairs, then each edge takes its pair's exclusion with its partner.  Rows
+// wider than eight compute the pairs' products twice rather than keep them.
+template <int DC, int V>
+__device__ __forceinline__ void row_outputs(float (&x)[DC][V], const float (&seed)[V]) {
+    static_assert(DC % 2 == 0 && DC >= 4, "rows are padded to pairs");
+    constexpr int n = DC / 2;
+    constexpr bool kKeep = DC <= 8;
+    float pr[kKeep ? n : 1][V], pre[n][V], run[V], e[V];
+#pragma unroll
+    for (int c = 0; c < V; ++c) pre[0][c] = seed[c];
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+        float *p = pr[kKeep ? i : 0];
+#pragma unroll
+        for (int c = 0; c < V; ++c) {
+            if (kKeep || i + 1 < n) p[c] = min_sign(x[2 * i][c], x[2 * i + 1][c]);
+            if (i + 1 < n) pre[i + 1][c] = min_sign(pre[i][c], p[c]);
+        }
+    }
+#pragma unroll
+    for (int i = n - 1; i >= 0; --i) {
+#pragma unroll
+        for (int c = 0; c < V; ++c) {
+            e[c] = i == n - 1 ? pre[i][c] : min_sign(pre[i][c], run[c]);
+            if (i > 0) {
+                const float p = kKeep ? pr[kKeep ? i : 0][c] : min_sign(x[2 * i][c], x[2 * i + 1][c]);
+                run[c] = i == n - 1 ? p : min_sign(run[c], p);
+            }
+            const float o = min_sign(x[2 * i + 1][c], e[c]);
+            x[2 * i + 1][c] = min_sign(x[2 * i][c], e[c]);
+            x[2 * i][c] = o;
+        }
+    }
+}
+
+// One row for V adjacent slots.  tauv = j*(S/V) + q; MQ: rank stride in V-slot groups.
+template <int DC, bool REG, int V>
+__device__ __forceinline__ void c_row(const LayoutMem &L, const TeamMem &T, int MQ, int lgQ, int tauv,
+                                      const float (&alpha)[V]) {
+    typedef typename VecF<V>::T VT;
+    VT *pv = reinterpret_cast<VT *>(T.m) + tauv;
+    const int deg = REG ? DC : (int)L.row_deg[tauv >> lgQ];
+    const unsigned sb = T.syn[(V * tauv) >> 5] >> ((V * tauv) & 31);
+    float x[DC][V], seed[V];
 #pragma unroll
     for (int k = 0; k < DC; ++k)
-        if (REG || k < t.deg) t.v[k] = t.p[k * MS];
+        if (REG || k < deg) {
+            vload<V>(x[k], pv + k * MQ);
+            vmul<V>(x[k], x[k], alpha);
+        } else {
+#pragma unroll
+            for (int c = 0; c < V; ++c) x[k][c] = __int_as_float(0x7f800000);
+        }
+    row_seed<V, true>(seed, sb);
+    row_outputs<DC, V>(x, seed);
+#pragma unroll
+    for (int k = 0; k < DC; ++k)
+        if (REG || k < deg) vstore<V>(pv + k * MQ, x[k]);
 }
 
-template <int DC, bool REG>
-__device__ __forceinline__ void c_compute_store(CTask<DC, REG> &t, int MS, float alpha) {
-    if (!t.on) return;
-    // m1 <= m2 are the two smallest |q_k| (equal on ties).  The message to
-    // edge k excludes k itself: alpha * m2 if |q_k| == m1, else alpha * m1
-    // (on a tie m2 == m1, so either choice gives the same value).
-    float m1 = __int_as_float(0x7f800000), m2 = m1;
-    unsigned sx = t.sall;
-#pragma unroll
-    for (int k = 0; k < DC; ++k) {
-        if (REG || k < t.deg) {
-            const float a = fabsf(t.v[k]);
-            m2 = fminf(m2, fmaxf(m1, a));
-            m1 = fminf(m1, a);
-            sx ^= __float_as_uint(t.v[k]);
-        }
-    }
-    // The row's sign product goes into both magnitudes (they are >= 0); each
-    // output then flips it by its own input's sign bit.
-    sx &= 0x80000000u;
-    const unsigned g1 = __float_as_uint(fminf(__fmul_rn(alpha, m1), kMagClamp)) | sx;
-    const unsigned g2 = __float_as_uint(fminf(__fmul_rn(alpha, m2), kMagClamp)) | sx;
-#pragma unroll
-    for (int k = 0; k < DC; ++k) {
-        if (REG || k < t.deg) {
-            const unsigned mag = (fabsf(t.v[k]) == m1) ? g2 : g1;
-            t.p[k * MS] = __uint_as_float(mag ^ (__float_as_uint(t.v[k]) & 0x80000000u));
-        }
-    }
-}
-
-// Rows (C phase) and columns (V phase) a thread handles per step: their
-// loads are all issued before any of their stores, for instruction-level
-// parallelism (the tasks of one step touch disjoint messages).
-// Teams with S >= 2 slots run the vector phases: a lane serves up to
-// BPSF_VEC adjacent slots (2 or 4); BPSF_PAIRS = 0 keeps one slot per lane.
-#ifndef BPSF_PAIRS
-#define BPSF_PAIRS 1
-#endif
-#ifndef BPSF_VEC
-#define BPSF_VEC 4
-#endif
-#ifndef BPSF_CU
-#define BPSF_CU 1
-#endif
-#ifndef BPSF_VU
-#define BPSF_VU 1
-#endif
-
-template <int DC, bool REG>
-__device__ __forceinline__ void c_phase(const CodeDev &cd, const LayoutMem &L, const TeamMem &T, int lgS, float alpha,
-                                        int tid, int nthreads) {
-    const int MS = cd.Mp << lgS;  // rank stride of the active layout
-    const int nt = cd.M << lgS;   // row tasks (rows M..Mp-1 of the stride are padding)
-    for (int tau = tid; tau < nt; tau += BPSF_CU * nthreads) {
-        CTask<DC, REG> t[BPSF_CU];
-#pragma unroll
-        for (int u = 0; u < BPSF_CU; ++u) c_load<DC, REG>(t[u], L, T, MS, lgS, tau + u * nthreads, tau + u * nthreads < nt);
-#pragma unroll
-        for (int u = 0; u < BPSF_CU; ++u) c_compute_store<DC, REG>(t[u], MS, alpha);
-    }
+template <int DC, bool REG, int V>
+__device__ __forceinline__ void c_phase(const CodeDev &cd, const LayoutMem &L, const TeamMem &T, int lgS,
+                                        const float (&alpha)[V], int tid, int nthreads) {
+    const int lgQ = lgS - (V == 4 ? 2 : V - 1);
+    const int MQ = cd.Mp << lgQ;  // rank stride of the active layout, in V-slot groups
+    const int nt = cd.M << lgQ;   // row tasks (rows M..Mp-1 of the stride are padding)
+    for (int tauv = tid; tauv < nt; tauv += nthreads) c_row<DC, REG, V>(L, T, MQ, lgQ, tauv, alpha);
 }
 
 // ---------------------------------------------------------------------------
@@ -281,250 +330,128 @@ __device__ __forceinline__ void c_phase(const CodeDev &cd, const LayoutMem &L, c
 // ascending check order:
 //   q_k   = l_ch + sum_{k' != k} r_k'   (left fold, ascending k'),
 //   l_out = l_ch + sum_k r_k            (left fold),  e_i = [l_out <= 0].
+// The C phase stores -r, so every step of a fold is one subtraction (the same
+// rounding), and the last one, taken the other way round, is -l_out: its sign
+// bit is set exactly when l_out > 0 (a zero comes out as +0), so the decision
+// is a sign bit and the slots' decisions are gathered by byte permutes.
+//
+// Lane l serves the V adjacent slots V*q .. V*q + V-1, q = l mod S/V.  Their
+// items are adjacent words, so one access of up to 128 bits moves all V slots'
+// messages; column tables, LLRs, addresses and loop control are shared, and
+// the V slots' residual-syndrome bits of a check sit in one word.  A slot of
+// the group that is not running is computed on its own stale data and its
+// messages are rewritten harmlessly (an install resets them); its
+// decision/flip word and syndrome bits are left alone.
 // ---------------------------------------------------------------------------
-template <int DVS>
-struct VTask {
-    uint16_t pos[DVS];  // edge positions r*Mp + j of the column's checks
-    float r[DVS];
-    float lc;
-    unsigned f;  // decision (bit 15) and flip count of (variable, slot)
-    int tau;
-    bool on;
-};
-
-// Task tau = i*S + s of the interleaved team layout: column i of slot s
-// (s is the lane's fixed slot).
-template <int DVS, int DVX, int FB>
-__device__ __forceinline__ void v_load(VTask<DVS> &t, const LayoutMem &L, const TeamMem &T, int lgS, int s, int tau,
-                                       bool on) {
-    t.on = on;
-    if (!on) return;
-    t.tau = tau;
-    const int i = tau >> lgS;
-    const uint16_t *vp = L.vpos + i * DVS;
-    if (DVS == 4) {
-        const uint2 raw = *reinterpret_cast<const uint2 *>(vp);
-        t.pos[0] = (uint16_t)(raw.x & 0xffffu);
-        t.pos[1] = (uint16_t)(raw.x >> 16);
-        t.pos[2] = (uint16_t)(raw.y & 0xffffu);
-        t.pos[3] = (uint16_t)(raw.y >> 16);
-    } else {
-#pragma unroll
-        for (int k = 0; k < DVS; ++k) t.pos[k] = vp[k];
-    }
-    t.lc = L.lch[i];
-    const float *ms = T.m + s;
-#pragma unroll
-    for (int k = 0; k < DVS; ++k)
-        if (DVX > 0 ? (k < DVX) : true)
-            t.r[k] = (DVX > 0 || t.pos[k] != 0xffffu) ? ms[(int)t.pos[k] << lgS] : 0.f;
-    t.f = (unsigned)flipw<FB>(T)[tau];
-}
-
-template <int DVS, int DVX, bool DEBUG, int FB>
-__device__ __forceinline__ void v_compute_store(const VTask<DVS> &t, const StreamDev &sd, const TeamMem &T, int lgS,
-                                                int s, unsigned initm) {
-    if (!t.on) return;
-    float *ms = T.m + s;
-    float lo;
-    if (DVX == 3) {
-        // Three checks: shared prefix l_ch + r0.
-        const float t0 = __fadd_rn(t.lc, t.r[0]);
-        const float q2 = __fadd_rn(t0, t.r[1]);
-        lo = __fadd_rn(q2, t.r[2]);
-        const float q1 = __fadd_rn(t0, t.r[2]);
-        const float q0 = __fadd_rn(__fadd_rn(t.lc, t.r[1]), t.r[2]);
-        ms[(int)t.pos[0] << lgS] = q0;
-        ms[(int)t.pos[1] << lgS] = q1;
-        ms[(int)t.pos[2] << lgS] = q2;
-    } else {
-#pragma unroll
-        for (int k = 0; k < DVS; ++k) {
-            if (t.pos[k] != 0xffffu) {
-                float acc = t.lc;
-#pragma unroll
-                for (int k2 = 0; k2 < DVS; ++k2)
-                    if (k2 != k && t.pos[k2] != 0xffffu) acc = __fadd_rn(acc, t.r[k2]);
-                ms[(int)t.pos[k] << lgS] = acc;
-            }
-        }
-        lo = t.lc;
-#pragma unroll
-        for (int k = 0; k < DVS; ++k)
-            if (t.pos[k] != 0xffffu) lo = __fadd_rn(lo, t.r[k]);
-    }
-    const unsigned ebit = (lo <= 0.f) ? 1u : 0u;
-    const int i = t.tau >> lgS;
-    if (DEBUG && ((initm >> s) & 1u) && sd.dbg.lout) sd.dbg.lout[T.st[s].shot * sd.code.N + i] = lo;
-    // The (variable, slot) flip word: decision and flip count (FlipW).
-    if (flip_dec<FB>(t.f) != ebit) {
-        flipw<FB>(T)[t.tau] = (typename FlipW<FB>::W)flip_bump<FB>(t.f);
-        // The residual syndrome s xor H e toggles at this column's checks
-        // (bit c*S + s of the team's residual-syndrome words).
-        const uint16_t *vc = sd.code.vchk + i * DVS;
-#pragma unroll
-        for (int k = 0; k < DVS; ++k) {
-            if (DVX > 0 ? (k < DVX) : (t.pos[k] != 0xffffu)) {
-                const int b = ((int)__ldg(vc + k) << lgS) + s;
-                atomicXor(&T.mism[b >> 5], 1u << (b & 31));
-            }
-        }
-    }
-}
-
-template <int DVS, int DVX, bool DEBUG, int FB>
-__device__ __forceinline__ void v_phase(const StreamDev &sd, const LayoutMem &L, const TeamMem &T, int lgS,
-                                        unsigned initm, int tid, int nthreads) {
-    const int total = sd.code.N << lgS;
-    const int s = tid & ((1 << lgS) - 1);
-    for (int tau = tid; tau < total; tau += BPSF_VU * nthreads) {
-        VTask<DVS> t[BPSF_VU];
-#pragma unroll
-        for (int u = 0; u < BPSF_VU; ++u)
-            v_load<DVS, DVX, FB>(t[u], L, T, lgS, s, tau + u * nthreads, tau + u * nthreads < total);
-#pragma unroll
-        for (int u = 0; u < BPSF_VU; ++u) v_compute_store<DVS, DVX, DEBUG, FB>(t[u], sd, T, lgS, s, initm);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Vector phases (S >= V, V = 2 or 4): lane l serves the V adjacent slots
-// V*q .. V*q + V-1, q = l mod S/V.  Their items are adjacent words, so one
-// 64- or 128-bit access moves all V slots' messages; column tables, LLRs,
-// addresses and loop control are shared, and the V slots' residual-syndrome
-// bits of a check sit in one word.  A slot of the group that is not running
-// is computed on its own stale data and its messages are rewritten
-// harmlessly (an install resets them); its decision/flip word and syndrome
-// bits are left alone.
-// ---------------------------------------------------------------------------
-template <int V> struct VecF;
-template <> struct VecF<2> { typedef float2 T; };
-template <> struct VecF<4> { typedef float4 T; };
 
 // The flip words of V adjacent slots packed in one integer U (slot c in the
-// c-th FB-byte field).  dmask: their decision bits as a mask with bit c for
-// slot c.  bump: toggle the decision and add one flip in the fields selected
-// by mask bm; a count is below max_iter before the increment, so no carry
-// leaves its field.
+// c-th FB-byte field).  on: the top bits of the fields of the slots in a mask.
+// diff: the top bits of the running slots' fields whose decision changes,
+// given -l_out.  bump: toggle the decision and add one flip there; a count is
+// below max_iter before the increment, so no carry leaves its field.  slots:
+// the changed slots as a mask.
 template <int FB, int V> struct FlipPack;
+template <int FB> struct FlipPack<FB, 1> {
+    typedef typename FlipW<FB>::W U;
+    typedef unsigned D;
+    static __device__ __forceinline__ D on(unsigned m) { return (m & 1u) << (8 * FB - 1); }
+    static __device__ __forceinline__ D diff(const float (&nl)[1], U w, D on) {
+        return (~(__float_as_uint(nl[0]) >> (32 - 8 * FB)) ^ (unsigned)w) & on;
+    }
+    static __device__ __forceinline__ bool any(D d) { return d != 0u; }
+    static __device__ __forceinline__ U bump(U w, D d) { return (U)(((unsigned)w ^ d) + (d >> (8 * FB - 1))); }
+    static __device__ __forceinline__ unsigned slots(D d) { return d >> (8 * FB - 1); }
+};
+__device__ __forceinline__ unsigned sign_halves(float a, float b) {
+    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0xffbb);
+}
 template <> struct FlipPack<2, 2> {
     typedef uint32_t U;
-    static __device__ __forceinline__ unsigned dmask(U w) { return ((w >> 15) & 1u) | ((w >> 30) & 2u); }
-    static __device__ __forceinline__ U bump(U w, unsigned bm) {
-        return (w ^ (((bm & 1u) << 15) | ((bm & 2u) << 30))) + ((bm & 1u) | ((bm & 2u) << 15));
-    }
+    typedef unsigned D;
+    static __device__ __forceinline__ D on(unsigned m) { return ((m & 1u) << 15) | ((m & 2u) << 30); }
+    static __device__ __forceinline__ D diff(const float (&nl)[2], U w, D on) { return (~sign_halves(nl[0], nl[1]) ^ w) & on; }
+    static __device__ __forceinline__ bool any(D d) { return d != 0u; }
+    static __device__ __forceinline__ U bump(U w, D d) { return (w ^ d) + (d >> 15); }
+    static __device__ __forceinline__ unsigned slots(D d) { return ((d >> 15) & 1u) | ((d >> 30) & 2u); }
 };
 template <> struct FlipPack<2, 4> {
     typedef uint2 U;
-    static __device__ __forceinline__ unsigned dmask(U w) {
-        return FlipPack<2, 2>::dmask(w.x) | (FlipPack<2, 2>::dmask(w.y) << 2);
+    typedef uint2 D;
+    typedef FlipPack<2, 2> H;
+    static __device__ __forceinline__ D on(unsigned m) { return make_uint2(H::on(m), H::on(m >> 2)); }
+    static __device__ __forceinline__ D diff(const float (&nl)[4], U w, D on) {
+        return make_uint2((~sign_halves(nl[0], nl[1]) ^ w.x) & on.x, (~sign_halves(nl[2], nl[3]) ^ w.y) & on.y);
     }
-    static __device__ __forceinline__ U bump(U w, unsigned bm) {
-        return make_uint2(FlipPack<2, 2>::bump(w.x, bm & 3u), FlipPack<2, 2>::bump(w.y, bm >> 2));
-    }
+    static __device__ __forceinline__ bool any(D d) { return (d.x | d.y) != 0u; }
+    static __device__ __forceinline__ U bump(U w, D d) { return make_uint2(H::bump(w.x, d.x), H::bump(w.y, d.y)); }
+    static __device__ __forceinline__ unsigned slots(D d) { return H::slots(d.x) | (H::slots(d.y) << 2); }
 };
 template <> struct FlipPack<1, 2> {
     typedef uint16_t U;
-    static __device__ __forceinline__ unsigned dmask(U w) {
-        const unsigned x = w;
-        return ((x >> 7) & 1u) | ((x >> 14) & 2u);
+    typedef unsigned D;
+    static __device__ __forceinline__ D on(unsigned m) { return ((m & 1u) << 7) | ((m & 2u) << 14); }
+    static __device__ __forceinline__ D diff(const float (&nl)[2], U w, D on) {
+        return (~__byte_perm(__float_as_uint(nl[0]), __float_as_uint(nl[1]), 0xfbfb) ^ (unsigned)w) & on;
     }
-    static __device__ __forceinline__ U bump(U w, unsigned bm) {
-        const unsigned sp = (bm & 1u) | ((bm & 2u) << 7);
-        return (U)(((unsigned)w ^ (sp << 7)) + sp);
-    }
+    static __device__ __forceinline__ bool any(D d) { return d != 0u; }
+    static __device__ __forceinline__ U bump(U w, D d) { return (U)(((unsigned)w ^ d) + (d >> 7)); }
+    static __device__ __forceinline__ unsigned slots(D d) { return ((d >> 7) & 1u) | ((d >> 14) & 2u); }
 };
 template <> struct FlipPack<1, 4> {
     typedef uint32_t U;
-    static __device__ __forceinline__ unsigned dmask(U w) {
-        return ((w >> 7) & 1u) | ((w >> 14) & 2u) | ((w >> 21) & 4u) | ((w >> 28) & 8u);
+    typedef unsigned D;
+    static __device__ __forceinline__ D on(unsigned m) { return ((m * 0x00204081u) & 0x01010101u) << 7; }
+    static __device__ __forceinline__ D diff(const float (&nl)[4], U w, D on) {
+        const unsigned p = __byte_perm(__float_as_uint(nl[0]), __float_as_uint(nl[1]), 0xfbfb);
+        const unsigned q = __byte_perm(__float_as_uint(nl[2]), __float_as_uint(nl[3]), 0xfbfb);
+        return (~__byte_perm(p, q, 0x5410) ^ w) & on;
     }
-    static __device__ __forceinline__ U bump(U w, unsigned bm) {
-        const unsigned sp = (bm & 1u) | ((bm & 2u) << 7) | ((bm & 4u) << 14) | ((bm & 8u) << 21);
-        return (w ^ (sp << 7)) + sp;
-    }
+    static __device__ __forceinline__ bool any(D d) { return d != 0u; }
+    static __device__ __forceinline__ U bump(U w, D d) { return (w ^ d) + (d >> 7); }
+    // Bits 7, 15, 23, 31 to 0..3: the four partial products meet no other in the top bits.
+    static __device__ __forceinline__ unsigned slots(D d) { return ((d >> 7) * 0x10204080u) >> 28; }
 };
 
-template <int V>
-__device__ __forceinline__ float &comp(typename VecF<V>::T &v, int c) { return reinterpret_cast<float *>(&v)[c]; }
-template <int V>
-__device__ __forceinline__ float compc(const typename VecF<V>::T &v, int c) {
-    return reinterpret_cast<const float *>(&v)[c];
-}
-
-template <int DC, bool REG, int V>
-__device__ __forceinline__ void c_row_vec(const LayoutMem &L, const TeamMem &T, int MQ, int lgQ, int tauv,
-                                          const float (&alpha)[V]) {
-    typedef typename VecF<V>::T VT;
-    VT *pv = reinterpret_cast<VT *>(T.m) + tauv;  // tauv = j*(S/V) + q
-    const int deg = REG ? DC : (int)L.row_deg[tauv >> lgQ];
-    const unsigned sb = T.syn[(V * tauv) >> 5] >> ((V * tauv) & 31);
-    VT v[DC];
+// The residual syndrome s xor H e toggles at the checks of column i for the
+// slots in bm (bit c*S + s of the team's residual-syndrome words).
+template <int DVS, int DVX>
+__device__ __forceinline__ void toggle_residual(const CodeDev &cd, const TeamMem &T, int lgS, int s0, int i,
+                                                unsigned bm) {
+    const uint16_t *vc = cd.vchk + i * DVS;
+    uint16_t chk[DVS];
+    if (DVS == 4) {
+        const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(vc));
+        chk[0] = (uint16_t)(raw.x & 0xffffu);
+        chk[1] = (uint16_t)(raw.x >> 16);
+        chk[2] = (uint16_t)(raw.y & 0xffffu);
+        chk[3] = (uint16_t)(raw.y >> 16);
+    } else {
 #pragma unroll
-    for (int k = 0; k < DC; ++k)
-        if (REG || k < deg) v[k] = pv[k * MQ];
-    float m1[V], m2[V];
-    unsigned sx[V];
-#pragma unroll
-    for (int c = 0; c < V; ++c) {
-        m1[c] = __int_as_float(0x7f800000);
-        m2[c] = m1[c];
-        sx[c] = ((sb >> c) & 1u) << 31;
+        for (int k = 0; k < DVS; ++k) chk[k] = __ldg(vc + k);
     }
 #pragma unroll
-    for (int k = 0; k < DC; ++k) {
-        if (REG || k < deg) {
-#pragma unroll
-            for (int c = 0; c < V; ++c) {
-                const float a = fabsf(compc<V>(v[k], c));
-                m2[c] = fminf(m2[c], fmaxf(m1[c], a));
-                m1[c] = fminf(m1[c], a);
-                sx[c] ^= __float_as_uint(compc<V>(v[k], c));
-            }
+    for (int k = 0; k < DVS; ++k) {
+        if (DVX > 0 ? (k < DVX) : (chk[k] != 0xffffu)) {
+            const int b = ((int)chk[k] << lgS) + s0;
+            atomicXor(&T.mism[b >> 5], bm << (b & 31));
         }
     }
-    unsigned g1[V], g2[V];
-#pragma unroll
-    for (int c = 0; c < V; ++c) {
-        sx[c] &= 0x80000000u;
-        g1[c] = __float_as_uint(fminf(__fmul_rn(alpha[c], m1[c]), kMagClamp)) | sx[c];
-        g2[c] = __float_as_uint(fminf(__fmul_rn(alpha[c], m2[c]), kMagClamp)) | sx[c];
-    }
-#pragma unroll
-    for (int k = 0; k < DC; ++k) {
-        if (REG || k < deg) {
-            VT o;
-#pragma unroll
-            for (int c = 0; c < V; ++c) {
-                const float x = compc<V>(v[k], c);
-                comp<V>(o, c) = __uint_as_float(((fabsf(x) == m1[c]) ? g2[c] : g1[c]) ^ (__float_as_uint(x) & 0x80000000u));
-            }
-            pv[k * MQ] = o;
-        }
-    }
-}
-
-template <int DC, bool REG, int V>
-__device__ __forceinline__ void c_phase_vec(const CodeDev &cd, const LayoutMem &L, const TeamMem &T, int lgS,
-                                            const float (&alpha)[V], int tid, int nthreads) {
-    const int lgQ = lgS - (V == 4 ? 2 : 1);
-    const int MQ = cd.Mp << lgQ;  // rank stride of the active layout, in V-slot groups
-    const int nt = cd.M << lgQ;   // row tasks (rows M..Mp-1 of the stride are padding)
-    for (int tauv = tid; tauv < nt; tauv += nthreads) c_row_vec<DC, REG, V>(L, T, MQ, lgQ, tauv, alpha);
 }
 
 template <int DVS, int DVX, bool DEBUG, int V, int FB>
-__device__ __forceinline__ void v_phase_vec(const StreamDev &sd, const LayoutMem &L, const TeamMem &T, int lgS,
-                                            unsigned onm, unsigned initm, int tid, int nthreads) {
+__device__ __forceinline__ void v_phase(const StreamDev &sd, const LayoutMem &L, const TeamMem &T, int lgS,
+                                        unsigned onm, unsigned initm, int tid, int nthreads) {
     typedef typename VecF<V>::T VT;
-    typedef typename FlipPack<FB, V>::U UT;
+    typedef FlipPack<FB, V> FP;
     const CodeDev &cd = sd.code;
-    const int lgQ = lgS - (V == 4 ? 2 : 1);
+    const int lgQ = lgS - (V == 4 ? 2 : V - 1);
     const int total = cd.N << lgQ;
     const int q = tid & ((1 << lgQ) - 1);
     const int s0 = V * q;
     VT *mv = reinterpret_cast<VT *>(T.m) + q;
-    UT *fv = reinterpret_cast<UT *>(T.flips);
+    typename FP::U *fv = reinterpret_cast<typename FP::U *>(T.flips);
+    const typename FP::D on = FP::on(onm);
+    constexpr int DV = DVX > 0 ? DVX : DVS;  // entries looked at (the rest of the table is padding)
     for (int tauv = tid; tauv < total; tauv += nthreads) {
         const int i = tauv >> lgQ;
         uint16_t pos[DVS];
@@ -539,236 +466,110 @@ __device__ __forceinline__ void v_phase_vec(const StreamDev &sd, const LayoutMem
 #pragma unroll
             for (int k = 0; k < DVS; ++k) pos[k] = vp[k];
         }
-        const float lc = L.lch[i];
-        VT r[DVS];
+        float lc[V];
+        {
+            const float l = L.lch[i];
 #pragma unroll
-        for (int k = 0; k < DVS; ++k)
-            if (DVX > 0 ? (k < DVX) : (pos[k] != 0xffffu)) r[k] = mv[(int)pos[k] << lgQ];
-        const UT fw = fv[tauv];
-        float lo[V];
-        if (DVX == 3) {
-            VT q0, q1, q2;
-#pragma unroll
-            for (int c = 0; c < V; ++c) {
-                const float t0 = __fadd_rn(lc, compc<V>(r[0], c));
-                const float a2 = __fadd_rn(t0, compc<V>(r[1], c));
-                lo[c] = __fadd_rn(a2, compc<V>(r[2], c));
-                comp<V>(q0, c) = __fadd_rn(__fadd_rn(lc, compc<V>(r[1], c)), compc<V>(r[2], c));
-                comp<V>(q1, c) = __fadd_rn(t0, compc<V>(r[2], c));
-                comp<V>(q2, c) = a2;
-            }
-            mv[(int)pos[0] << lgQ] = q0;
-            mv[(int)pos[1] << lgQ] = q1;
-            mv[(int)pos[2] << lgQ] = q2;
-        } else {
-#pragma unroll
-            for (int k = 0; k < DVS; ++k) {
-                if (pos[k] != 0xffffu) {
-                    VT acc;
-#pragma unroll
-                    for (int c = 0; c < V; ++c) comp<V>(acc, c) = lc;
-#pragma unroll
-                    for (int k2 = 0; k2 < DVS; ++k2)
-                        if (k2 != k && pos[k2] != 0xffffu)
-#pragma unroll
-                            for (int c = 0; c < V; ++c) comp<V>(acc, c) = __fadd_rn(compc<V>(acc, c), compc<V>(r[k2], c));
-                    mv[(int)pos[k] << lgQ] = acc;
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < V; ++c) lo[c] = lc;
-#pragma unroll
-            for (int k = 0; k < DVS; ++k)
-                if (pos[k] != 0xffffu)
-#pragma unroll
-                    for (int c = 0; c < V; ++c) lo[c] = __fadd_rn(lo[c], compc<V>(r[k], c));
+            for (int c = 0; c < V; ++c) lc[c] = l;
         }
-        // Decision (bit 15) and flip count of each slot's 16-bit word: the
-        // running slots whose decision changed, as a mask.
-        unsigned em = 0;
+        // A missing entry reads as 0: subtracting +0 changes nothing.
+        float r[DV][V];
 #pragma unroll
-        for (int c = 0; c < V; ++c) {
-            em |= ((lo[c] <= 0.f) ? 1u : 0u) << c;
-            if (DEBUG && sd.dbg.lout && ((onm >> c) & 1u) && ((initm >> (s0 + c)) & 1u))
-                sd.dbg.lout[T.st[s0 + c].shot * cd.N + i] = lo[c];
-        }
-        const unsigned bm = (em ^ FlipPack<FB, V>::dmask(fw)) & onm;
-        if (bm) {
-            fv[tauv] = FlipPack<FB, V>::bump(fw, bm);
-            const uint16_t *vc = cd.vchk + i * DVS;
+        for (int k = 0; k < DV; ++k) {
+            if (DVX > 0 || pos[k] != 0xffffu) {
+                vload<V>(r[k], mv + ((int)pos[k] << lgQ));
+            } else {
 #pragma unroll
-            for (int k = 0; k < DVS; ++k) {
-                if (DVX > 0 ? (k < DVX) : (pos[k] != 0xffffu)) {
-                    const int b = ((int)__ldg(vc + k) << lgS) + s0;
-                    atomicXor(&T.mism[b >> 5], bm << (b & 31));
-                }
+                for (int c = 0; c < V; ++c) r[k][c] = 0.f;
             }
+        }
+        const typename FP::U fw = fv[tauv];
+        // pre = l_ch + r_0 + .. + r_{k-1}; q_k goes on from there without r_k.
+        float pre[V], nl[V];
+#pragma unroll
+        for (int c = 0; c < V; ++c) pre[c] = lc[c];
+#pragma unroll
+        for (int k = 0; k < DV; ++k) {
+            float acc[V];
+#pragma unroll
+            for (int c = 0; c < V; ++c) acc[c] = pre[c];
+#pragma unroll
+            for (int k2 = k + 1; k2 < DV; ++k2) vsub<V>(acc, acc, r[k2]);
+            if (k + 1 < DV)
+                vsub<V>(pre, pre, r[k]);
+            else
+                vsub<V>(nl, r[k], pre);  // -l_out
+            if (DVX > 0 || pos[k] != 0xffffu) vstore<V>(mv + ((int)pos[k] << lgQ), acc);
+        }
+        if (DEBUG && sd.dbg.lout) {
+#pragma unroll
+            for (int c = 0; c < V; ++c)
+                if (((onm >> c) & 1u) && ((initm >> (s0 + c)) & 1u))
+                    sd.dbg.lout[T.st[s0 + c].shot * cd.N + i] = __fsub_rn(0.f, nl[c]);
+        }
+        const typename FP::D d = FP::diff(nl, fw, on);
+        if (FP::any(d)) {
+            fv[tauv] = FP::bump(fw, d);
+            toggle_residual<DVS, DVX>(cd, T, lgS, s0, i, FP::slots(d));
         }
     }
 }
 
 // ---------------------------------------------------------------------------
-// Layered schedule (one slot per lane).  Layer by layer (rows of a layer
-// share no variable, so they run in parallel and in any order), each row j
-// of slot s: q_k = L_i - r_k for its edges k (i = the k-th variable of the
-// row, r_k its C2V message from the previous iteration), new C2V messages
-// from the q_k by Eq. (c2v) as in the C phase, then L_i = q_k + r_k.  After
-// all layers L is the posterior: hard decision, flip counters and residual
-// syndrome as in the V phase.
+// Layered schedule.  Layer by layer (rows of a layer share no variable, so
+// they run in parallel and in any order), each row j of slot s:
+// q_k = L_i - r_k for its edges k (i = the k-th variable of the row, r_k its
+// C2V message from the previous iteration), new C2V messages from the q_k by
+// Eq. (c2v) as in the C phase, then L_i = q_k + r_k.  After all layers L is the
+// posterior: hard decision, flip counters and residual syndrome as in the V
+// phase.  A lane serves V adjacent slots; slots of the group that are not
+// running compute on stale values, and their results are never read (a slot's
+// messages and posterior are set up again when it takes its next item).
 // ---------------------------------------------------------------------------
-template <int DC>
-__device__ __forceinline__ void layered_row(const CodeDev &cd, const LayoutMem &L, const TeamMem &T, int lgS, int j,
-                                            int s, float alpha) {
-    const int S = 1 << lgS, M = cd.Mp;  // rank stride of the active layout
-    const int deg = (int)L.row_deg[j];
-    float q[DC];
-    int vi[DC];
-    float *mj = T.m + (j << lgS) + s;  // edge k of row j at ((k*M + j)*S + s)
-#pragma unroll
-    for (int k = 0; k < DC; ++k) {
-        if (k < deg) {
-            vi[k] = (int)__ldg(cd.pos_var + k * M + j);
-            q[k] = __fsub_rn(T.post[(vi[k] << lgS) + s], mj[k * M * S]);
-        }
-    }
-    float m1 = __int_as_float(0x7f800000), m2 = m1;
-    unsigned sx = ((T.syn[((j << lgS) + s) >> 5] >> (((j << lgS) + s) & 31)) & 1u) << 31;
-#pragma unroll
-    for (int k = 0; k < DC; ++k) {
-        if (k < deg) {
-            const float a = fabsf(q[k]);
-            m2 = fminf(m2, fmaxf(m1, a));
-            m1 = fminf(m1, a);
-            sx ^= __float_as_uint(q[k]);
-        }
-    }
-    sx &= 0x80000000u;
-    const unsigned g1 = __float_as_uint(fminf(__fmul_rn(alpha, m1), kMagClamp)) | sx;
-    const unsigned g2 = __float_as_uint(fminf(__fmul_rn(alpha, m2), kMagClamp)) | sx;
-#pragma unroll
-    for (int k = 0; k < DC; ++k) {
-        if (k < deg) {
-            const float r = __uint_as_float(((fabsf(q[k]) == m1) ? g2 : g1) ^ (__float_as_uint(q[k]) & 0x80000000u));
-            mj[k * M * S] = r;
-            T.post[(vi[k] << lgS) + s] = __fadd_rn(q[k], r);
-        }
-    }
-}
-
-template <int DC, int DVS, int DVX, bool DEBUG, int FB>
-__device__ __forceinline__ void layered_iteration(const StreamDev &sd, const LayoutMem &L, const TeamMem &T, int lgS,
-                                                  bool lane_on, float alpha, unsigned initm, int tid, int nthreads,
-                                                  int W, int bar_id) {
-    const CodeDev &cd = sd.code;
-    const int S = 1 << lgS;
-    const int s = tid & (S - 1);
-    for (int layer = 0; layer < cd.n_layers; ++layer) {
-        const int r0 = (int)__ldg(cd.layer_ptr + layer), r1 = (int)__ldg(cd.layer_ptr + layer + 1);
-        const int total = (r1 - r0) << lgS;
-        if (lane_on)
-            for (int tau = tid; tau < total; tau += nthreads)
-                layered_row<DC>(cd, L, T, lgS, (int)__ldg(cd.layer_rows + r0 + (tau >> lgS)), s, alpha);
-        team_sync(W, bar_id);
-    }
-    if (!lane_on) return;
-    const int N = cd.N;
-    for (int tau = tid; tau < (N << lgS); tau += nthreads) {
-        const int i = tau >> lgS;
-        const float lo = T.post[tau];
-        const unsigned ebit = (lo <= 0.f) ? 1u : 0u;
-        if (DEBUG && ((initm >> s) & 1u) && sd.dbg.lout) sd.dbg.lout[T.st[s].shot * N + i] = lo;
-        const unsigned f = (unsigned)flipw<FB>(T)[tau];
-        if (flip_dec<FB>(f) != ebit) {
-            flipw<FB>(T)[tau] = (typename FlipW<FB>::W)flip_bump<FB>(f);
-            const uint16_t *vc = cd.vchk + i * DVS;
-#pragma unroll
-            for (int k = 0; k < DVS; ++k) {
-                const int c = (int)__ldg(vc + k);
-                if (DVX > 0 ? (k < DVX) : (c != 0xffff)) {
-                    const int b = (c << lgS) + s;
-                    atomicXor(&T.mism[b >> 5], 1u << (b & 31));
-                }
-            }
-        }
-    }
-}
-
-// Layered schedule with V adjacent slots per lane (the slots' words are
-// adjacent in the interleaved layout): the same row and posterior updates as
-// layered_row, on V slots at once with vector loads and stores.  Slots of the
-// group that are not running compute on stale values; their results are
-// never read (a slot's messages and posterior are set up again when it takes
-// its next item).
-template <int DC, int V>
-__device__ __forceinline__ void layered_row_vec(const CodeDev &cd, const LayoutMem &L, const TeamMem &T, int lgQ, int j,
-                                                int q, const float (&alpha)[V]) {
+template <int DC, bool REG, int V>
+__device__ __forceinline__ void layered_row(const CodeDev &cd, const LayoutMem &L, const TeamMem &T, int lgQ, int j,
+                                            int q, const float (&alpha)[V]) {
     typedef typename VecF<V>::T VT;
     const int M = cd.Mp, MQ = cd.Mp << lgQ;  // rank stride of the active layout (in V-slot groups: MQ)
-    const int deg = (int)L.row_deg[j];
+    const int deg = REG ? DC : (int)L.row_deg[j];
     VT *mj = reinterpret_cast<VT *>(T.m) + (j << lgQ) + q;  // edge k of row j at (k*M + j)*Q + q
-    VT *pv = reinterpret_cast<VT *>(T.post) + q;             // posterior of variable i at i*Q + q
-    VT qv[DC];
+    VT *pv = reinterpret_cast<VT *>(T.post) + q;            // posterior of variable i at i*Q + q
+    float qv[DC][V], x[DC][V], seed[V];
 #pragma unroll
     for (int k = 0; k < DC; ++k) {
-        if (k < deg) {
-            const VT lp = pv[(int)__ldg(cd.pos_var + k * M + j) << lgQ], r = mj[k * MQ];
+        if (REG || k < deg) {
+            float lp[V], r[V];
+            vload<V>(lp, pv + ((int)__ldg(cd.pos_var + k * M + j) << lgQ));
+            vload<V>(r, mj + k * MQ);
+            vsub<V>(qv[k], lp, r);
+            vmul<V>(x[k], qv[k], alpha);
+        } else {
 #pragma unroll
-            for (int c = 0; c < V; ++c) comp<V>(qv[k], c) = __fsub_rn(compc<V>(lp, c), compc<V>(r, c));
+            for (int c = 0; c < V; ++c) x[k][c] = __int_as_float(0x7f800000);
         }
     }
-    const int b0 = (j << (lgQ + (V == 4 ? 2 : 1))) + V * q;  // syndrome bit of row j, first slot of the group
-    const unsigned sb = T.syn[b0 >> 5] >> (b0 & 31);
-    float m1[V], m2[V];
-    unsigned sx[V];
-#pragma unroll
-    for (int c = 0; c < V; ++c) {
-        m1[c] = __int_as_float(0x7f800000);
-        m2[c] = m1[c];
-        sx[c] = ((sb >> c) & 1u) << 31;
-    }
+    const int b0 = V * ((j << lgQ) + q);  // syndrome bit of row j, first slot of the group
+    row_seed<V, false>(seed, T.syn[b0 >> 5] >> (b0 & 31));
+    row_outputs<DC, V>(x, seed);
 #pragma unroll
     for (int k = 0; k < DC; ++k) {
-        if (k < deg) {
-#pragma unroll
-            for (int c = 0; c < V; ++c) {
-                const float a = fabsf(compc<V>(qv[k], c));
-                m2[c] = fminf(m2[c], fmaxf(m1[c], a));
-                m1[c] = fminf(m1[c], a);
-                sx[c] ^= __float_as_uint(compc<V>(qv[k], c));
-            }
-        }
-    }
-    unsigned g1[V], g2[V];
-#pragma unroll
-    for (int c = 0; c < V; ++c) {
-        sx[c] &= 0x80000000u;
-        g1[c] = __float_as_uint(fminf(__fmul_rn(alpha[c], m1[c]), kMagClamp)) | sx[c];
-        g2[c] = __float_as_uint(fminf(__fmul_rn(alpha[c], m2[c]), kMagClamp)) | sx[c];
-    }
-#pragma unroll
-    for (int k = 0; k < DC; ++k) {
-        if (k < deg) {
-            VT r, np;
-#pragma unroll
-            for (int c = 0; c < V; ++c) {
-                const float x = compc<V>(qv[k], c);
-                comp<V>(r, c) = __uint_as_float(((fabsf(x) == m1[c]) ? g2[c] : g1[c]) ^ (__float_as_uint(x) & 0x80000000u));
-                comp<V>(np, c) = __fadd_rn(x, compc<V>(r, c));
-            }
-            mj[k * MQ] = r;
-            pv[(int)__ldg(cd.pos_var + k * M + j) << lgQ] = np;  // the variable is read again: fewer live registers
+        if (REG || k < deg) {
+            float np[V];
+            vadd<V>(np, qv[k], x[k]);
+            vstore<V>(mj + k * MQ, x[k]);
+            vstore<V>(pv + ((int)__ldg(cd.pos_var + k * M + j) << lgQ), np);  // read again: fewer live registers
         }
     }
 }
 
 template <int DC, int DVS, int DVX, bool DEBUG, int V, int FB>
-__device__ __forceinline__ void layered_iteration_vec(const StreamDev &sd, const LayoutMem &L, const TeamMem &T,
-                                                      int lgS, unsigned onm, const float (&alpha)[V], unsigned initm,
-                                                      int tid, int nthreads, int W, int bar_id) {
+__device__ __forceinline__ void layered_iteration(const StreamDev &sd, const LayoutMem &L, const TeamMem &T, int lgS,
+                                                  unsigned onm, const float (&alpha)[V], unsigned initm, int tid,
+                                                  int nthreads, int W, int bar_id) {
     typedef typename VecF<V>::T VT;
-    typedef typename FlipPack<FB, V>::U UT;
+    typedef FlipPack<FB, V> FP;
     const CodeDev &cd = sd.code;
-    const int lgQ = lgS - (V == 4 ? 2 : 1);
+    const int lgQ = lgS - (V == 4 ? 2 : V - 1);
     const int q = tid & ((1 << lgQ) - 1);  // the lane's slot group: slots V*q .. V*q + V-1
     const int s0 = V * q;
     for (int layer = 0; layer < cd.n_layers; ++layer) {
@@ -776,36 +577,29 @@ __device__ __forceinline__ void layered_iteration_vec(const StreamDev &sd, const
         const int total = (r1 - r0) << lgQ;
         if (onm)
             for (int tauv = tid; tauv < total; tauv += nthreads)
-                layered_row_vec<DC, V>(cd, L, T, lgQ, (int)__ldg(cd.layer_rows + r0 + (tauv >> lgQ)), q, alpha);
+                layered_row<DC, (DVX > 0), V>(cd, L, T, lgQ, (int)__ldg(cd.layer_rows + r0 + (tauv >> lgQ)), q, alpha);
         team_sync(W, bar_id);
     }
     if (!onm) return;
     const int N = cd.N;
     const VT *pv = reinterpret_cast<const VT *>(T.post);
-    UT *fv = reinterpret_cast<UT *>(T.flips);
+    typename FP::U *fv = reinterpret_cast<typename FP::U *>(T.flips);
+    const typename FP::D on = FP::on(onm);
     for (int tauv = tid; tauv < (N << lgQ); tauv += nthreads) {
         const int i = tauv >> lgQ;
-        const VT lo = pv[tauv];
-        const UT fw = fv[tauv];
-        unsigned em = 0;
+        float lo[V], nl[V];
+        vload<V>(lo, pv + tauv);
+        const typename FP::U fw = fv[tauv];
 #pragma unroll
         for (int c = 0; c < V; ++c) {
-            em |= ((compc<V>(lo, c) <= 0.f) ? 1u : 0u) << c;
+            nl[c] = __fsub_rn(0.f, lo[c]);  // a zero of either sign comes out as +0: decided 1
             if (DEBUG && sd.dbg.lout && ((onm >> c) & 1u) && ((initm >> (s0 + c)) & 1u))
-                sd.dbg.lout[T.st[s0 + c].shot * N + i] = compc<V>(lo, c);
+                sd.dbg.lout[T.st[s0 + c].shot * N + i] = lo[c];
         }
-        const unsigned bm = (em ^ FlipPack<FB, V>::dmask(fw)) & onm;
-        if (bm) {
-            fv[tauv] = FlipPack<FB, V>::bump(fw, bm);
-            const uint16_t *vc = cd.vchk + i * DVS;
-#pragma unroll
-            for (int k = 0; k < DVS; ++k) {
-                const int c = (int)__ldg(vc + k);
-                if (DVX > 0 ? (k < DVX) : (c != 0xffff)) {
-                    const int b = (c << lgS) + s0;
-                    atomicXor(&T.mism[b >> 5], bm << (b & 31));
-                }
-            }
+        const typename FP::D d = FP::diff(nl, fw, on);
+        if (FP::any(d)) {
+            fv[tauv] = FP::bump(fw, d);
+            toggle_residual<DVS, DVX>(cd, T, lgS, s0, i, FP::slots(d));
         }
     }
 }
@@ -1031,12 +825,11 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
     const int lane = tid & 31, wt = tid >> 5, nthreads = 32 * W;
     const CodeDev &cd = sd.code;
     const int lgS = __ffs(S) - 1;
-    const int my_slot = lane & (S - 1);             // the slot this lane serves in every phase
     const int n_rwords = ((cd.M << lgS) + 31) >> 5;  // residual-syndrome words of the team
     const unsigned full = S >= 32 ? 0xffffffffu : ((1u << S) - 1u);
-    constexpr bool kVec = BPSF_PAIRS && DC <= 16;  // the widest rows keep one slot per lane (registers)
+    constexpr bool kVec = DC <= 16;  // the widest rows keep one slot per lane (registers)
     // Four slots per lane: exact-degree rows with the full register budget (one block).
-    constexpr bool kVec4 = kVec && MINB == 1 && DVX == 3 && BPSF_VEC >= 4;
+    constexpr bool kVec4 = kVec && MINB == 1 && DVX == 3;
     // Layered schedule: vector lanes in the full-register instances only.
     constexpr bool kLayV2 = LAY && kVec && MINB == 1 && DC <= 6, kLayV4 = kLayV2 && kVec4;
     const bool lay = LAY && cd.layered;
@@ -1153,42 +946,33 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
 #pragma unroll
         for (int c = 0; c < 4; ++c)
             al[c] = adaptive && c < vs ? damping(cd, tt - T.st[s0 + c].start + 1) : cd.alpha;
+        const unsigned onm = (run >> s0) & ((1u << vs) - 1u);  // the lane's running slots
         if (lay) {
             if (kLayV4 && vs == 4) {
-                float a4[4] = {al[0], al[1], al[2], al[3]};
-                layered_iteration_vec<DC, DVS, DVX, DEBUG, 4, FB>(sd, L, T, lgS, (run >> s0) & 0xfu, a4, initm, tid,
-                                                              nthreads, W, bar_id);
+                layered_iteration<DC, DVS, DVX, DEBUG, 4, FB>(sd, L, T, lgS, onm, al, initm, tid, nthreads, W, bar_id);
             } else if (kLayV2 && vs == 2) {
-                float a2[2] = {al[0], al[1]};
-                layered_iteration_vec<DC, DVS, DVX, DEBUG, 2, FB>(sd, L, T, lgS, (run >> s0) & 0x3u, a2, initm, tid,
-                                                              nthreads, W, bar_id);
+                const float a2[2] = {al[0], al[1]};
+                layered_iteration<DC, DVS, DVX, DEBUG, 2, FB>(sd, L, T, lgS, onm, a2, initm, tid, nthreads, W, bar_id);
             } else {
-                const bool lane_on = (run >> my_slot) & 1u;
-                layered_iteration<DC, DVS, DVX, DEBUG, FB>(sd, L, T, lgS, lane_on, al[0], initm, tid, nthreads, W,
-                                                       bar_id);
+                const float a1[1] = {al[0]};
+                layered_iteration<DC, DVS, DVX, DEBUG, 1, FB>(sd, L, T, lgS, onm, a1, initm, tid, nthreads, W, bar_id);
             }
-            team_sync(W, bar_id);
         } else if (kVec4 && vs == 4) {
-            const unsigned onm = (run >> s0) & 0xfu;
-            float a4[4] = {al[0], al[1], al[2], al[3]};
-            if (onm) c_phase_vec<DC, (DVX > 0), 4>(cd, L, T, lgS, a4, tid, nthreads);
+            if (onm) c_phase<DC, (DVX > 0), 4>(cd, L, T, lgS, al, tid, nthreads);
             team_sync(W, bar_id);
-            if (onm) v_phase_vec<DVS, DVX, DEBUG, 4, FB>(sd, L, T, lgS, onm, initm, tid, nthreads);
-            team_sync(W, bar_id);
+            if (onm) v_phase<DVS, DVX, DEBUG, 4, FB>(sd, L, T, lgS, onm, initm, tid, nthreads);
         } else if (kVec && vs == 2) {
-            const unsigned onm = (run >> s0) & 0x3u;
-            float a2[2] = {al[0], al[1]};
-            if (onm) c_phase_vec<DC, (DVX > 0), 2>(cd, L, T, lgS, a2, tid, nthreads);
+            const float a2[2] = {al[0], al[1]};
+            if (onm) c_phase<DC, (DVX > 0), 2>(cd, L, T, lgS, a2, tid, nthreads);
             team_sync(W, bar_id);
-            if (onm) v_phase_vec<DVS, DVX, DEBUG, 2, FB>(sd, L, T, lgS, onm, initm, tid, nthreads);
-            team_sync(W, bar_id);
+            if (onm) v_phase<DVS, DVX, DEBUG, 2, FB>(sd, L, T, lgS, onm, initm, tid, nthreads);
         } else {
-            const bool lane_on = (run >> my_slot) & 1u;
-            if (lane_on) c_phase<DC, (DVX > 0)>(cd, L, T, lgS, al[0], tid, nthreads);
+            const float a1[1] = {al[0]};
+            if (onm) c_phase<DC, (DVX > 0), 1>(cd, L, T, lgS, a1, tid, nthreads);
             team_sync(W, bar_id);
-            if (lane_on) v_phase<DVS, DVX, DEBUG, FB>(sd, L, T, lgS, initm, tid, nthreads);
-            team_sync(W, bar_id);
+            if (onm) v_phase<DVS, DVX, DEBUG, 1, FB>(sd, L, T, lgS, onm, initm, tid, nthreads);
         }
+        team_sync(W, bar_id);
         // Decision, in every warp: slot s owns bits s, s + S, s + 2S, ... of
         // every residual-syndrome word, so OR-folding the words down to S
         // bits leaves bit s set iff slot s's residual syndrome is not zero.
