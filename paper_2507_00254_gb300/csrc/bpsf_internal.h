@@ -74,7 +74,7 @@ struct CodeDev {
 struct StreamCounters {
     unsigned long long shot_next;    // next unclaimed shot
     unsigned long long init_done;    // initial runs finished
-    unsigned long long ticket_next;  // trial tickets claimed
+    unsigned long long rec_head;     // first failure whose record may have unclaimed trials
     unsigned long long iters_total;  // iterations run (all runs)
     unsigned long long trial_runs;   // trial runs finished
     unsigned long long rec_count;    // failed shots published
@@ -90,8 +90,8 @@ static_assert(sizeof(StreamCounters) == 128, "counter block is two 64-byte lines
 // order.  The team whose initial run fails claims the next failure number q
 // (rec_count), checks that record q % cap is free, writes Phi, the syndrome,
 // an empty selection and the shot's provisional output, and then publishes
-// it (qseq = q + 1); trial tickets walk the failure numbers, and the last
-// trial of a shot frees its record (qseq = 0).  A batch's ring has at least
+// it (qseq = q + 1); trials are claimed about in failure order, and the last
+// trial of a shot frees its record (qseq gets the kRecFree bit).  A batch's ring has at least
 // as many records as the batch has shots, so it never wraps within a launch
 // and the records are written densely in failure order; a server's ring has
 // at least its admitted shots (so it wraps only over freed records).  A
@@ -105,15 +105,20 @@ static_assert(sizeof(StreamCounters) == 128, "counter block is two 64-byte lines
 // minimum is then the smallest key's own word, whatever order the trials
 // finish in, with no lock.
 struct Records {
-    unsigned long long *qseq;   // cap: q + 1 while the record holds failure q, 0 when free
+    unsigned long long *qseq;   // cap: q + 1 while the record holds failure q, with kRecFree after; 0: never used
     long long *qshot;           // cap: the failed shot
-    unsigned int *done;         // cap: its trials finished
+    unsigned int *done;         // cap: its trials finished (kDoneBits bits); above them, its trials claimed
     unsigned long long *best;   // cap: min over converged trials of key << 32 | iterations
     unsigned long long *win;    // cap x Wn: min over converged trials of key << 32 | correction word
     int32_t *phi;               // cap x w
     uint32_t *synd;             // cap x Ws: the shot's syndrome
     long long cap;              // records in the ring (a power of two)
 };
+
+// Trials finished: n_trials <= 4096.  Claims past a record's end are at most 32
+// for each block of the launch, far below the 2^19 that the rest can count.
+constexpr int kDoneBits = 13;
+constexpr unsigned long long kRecFree = 1ull << 63;
 
 constexpr int kSelKeyBits = 28;  // weight (16 bits, N <= 65535) above a 12-bit list index (n_trials <= 4096)
 

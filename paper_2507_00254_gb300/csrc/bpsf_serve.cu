@@ -238,7 +238,9 @@ extern "C" bpsf_status bpsf_serve_start(bpsf_server **out, bpsf_ctx *const *code
         if (e != cudaSuccess) break;
         // A ring of failed-shot records (failed shots in flight never
         // outnumber admitted shots), all free.
-        const long long RR = bpsf_record_ring((long long)R);
+        // A claim reads a record's number and its count one after the other: with
+        // at least 1024 records none is reused in between.
+        const long long RR = bpsf_record_ring(std::max<long long>((long long)R, 1024));
         e = cudaMalloc(&sc.d_rec, bpsf_records_bytes(RR, x->p.w, x->Ws, x->Wn, 16));
         if (e != cudaSuccess) break;
         sc.rec = bpsf_records_carve(sc.d_rec, RR, x->p.w, x->Ws, x->Wn, 16);
