@@ -254,6 +254,11 @@ bpsf_status bpsf_sync(bpsf_ctx *ctx, void *stream);
  * layered schedule, a kernel instance with one-byte flip counters makes
  * room for shapes that two-byte counters do not fit (for example 13 teams of
  * 8 slots on [[144,12,12]]).
+ * Small batches (up to about 1.5 * 10^6 shots times columns in a launch, for
+ * example 10^4 shots of [[144,12,12]]) of codes of row weight 6 and column
+ * weight 3 without the layered schedule run with a lane per column instead, on
+ * a shape of their own, unless blocks_per_sm is given.  Results do not depend
+ * on it.
  */
 typedef struct {
     int32_t warps_per_team;  /* 1, 2, 4 or 8 */

@@ -148,8 +148,56 @@ static cudaError_t blocks_per_sm(const void *fn, int block, int smem, int *occ) 
     return e;
 }
 
+// Small launches of exact (6, 4, 3) codes run on the column path: a team of
+// ceil(N / 32) warps whose lanes hold a column each.  Its iteration is several
+// times shorter than that of a warp that serves a few slots, and it has fewer
+// slots; so it wins while a launch is short against a failed shot's chain of
+// iterations (0.6 against 1.8 us for each with few runs in flight), up to about
+// 1.5 * 10^6 columns of shots.  [[144]] at p = 0.05, column path against tuned
+// teams: 16 shots (p = 0.08) 0.24 / 0.37 ms, 300 0.16 / 0.34, 3000 0.36 /
+// 0.47, 30 000 2.7 / 1.85; at p = 0.02 10 000 shots 0.20 / 0.37, 100 000 0.96 /
+// 0.75; [[72]], 10 000 0.23 / 0.29; [[288]], 3000 0.62 / 0.68.
+// One slot per team where even all trials of all shots would not fill those
+// (100 iterations of one shot 70 against 86 us), else four.  A shape with a
+// given number of blocks per SM is taken at its word.
+constexpr long long kColumnShots = 1500000;
+
+static void plan_columns(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, const long long *shots,
+                         int base, bpsf_plan *out, int *variant, int *B, int *smem, long long *grid_max, int Q) {
+    if (kernel_variant_columns(base, 2) < 0) return;
+    long long work = 0;
+    int fb = 1;
+    for (int k = 0; k < n_codes; ++k) {
+        if ((codes[k]->N + 31) / 32 > kMaxColumnWarps || codes[k]->team_only || tunes[k].blocks_per_sm > 0) return;
+        if (codes[k]->p.max_iter > 127) fb = 2;
+        if (shots[k] > kColumnShots) return;
+        work += shots[k] * codes[k]->N;
+    }
+    if (work > kColumnShots) return;
+    const int vstride = kernel_variant_dv(base);
+    int warps = 0, bytes = 0;
+    long long blocks = 0;
+    for (int k = 0; k < n_codes; ++k) {
+        const bpsf_ctx *c = codes[k];
+        const int W = (c->N + 31) / 32, teams = std::min(kMaxNamedTeams, kMaxColumnWarps / W);
+        const long long runs = shots[k] * (1 + c->n_trials);
+        const int S = runs <= (long long)teams * c->sm_count ? 1 : 4;
+        out->W_code[k] = W;
+        out->S_code[k] = S;
+        out->teams_code[k] = teams;
+        blocks += (runs + teams * S - 1) / (teams * S);
+        warps = std::max(warps, W * teams);
+        bytes = std::max(bytes, block_smem_bytes(c->M, c->N, c->code.lay[layout_index(S)].P, c->Ws, vstride, S, teams, Q,
+                                                 0, fb, true));
+    }
+    *variant = kernel_variant_columns(base, fb);
+    *B = warps;
+    *smem = bytes;
+    *grid_max = std::max(1ll, blocks);
+}
+
 bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, bool debug,
-                           bpsf_plan *out, bool shrink) {
+                           bpsf_plan *out, bool shrink, const long long *shots) {
     // One kernel variant must fit every code of the launch.
     bool all_regular = true, layered = false;
     int dc = 0, dv = 0, B = 0, bps = 0;
@@ -224,6 +272,9 @@ bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tunin
             any_exact = any_exact || (codes[k]->regular && codes[k]->dc_max == 6 && codes[k]->dv_max == 3);
         if (any_exact) variant = kernel_variant_mixed(variant);
     }
+    long long grid_max = 1ll << 30;
+    if (shots && all_regular && !layered)
+        plan_columns(codes, n_codes, tunes, shots, kernel_variant(-dc, dv), out, &variant, &B, &smem, &grid_max, Q);
     bpsf_status st = bpsf_ensure_kernel_attrs(variant, c0->smem_optin);
     if (st != BPSF_OK) return st;
     const int block = 32 * (B + 1);
@@ -251,7 +302,7 @@ bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tunin
     out->Q = Q;
     out->block = block;
     out->smem = smem;
-    out->grid = occ * c0->sm_count;
+    out->grid = (int)std::min<long long>((long long)occ * c0->sm_count, grid_max);
     return BPSF_OK;
 }
 
@@ -497,6 +548,16 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     for (int e = 0; e < nnz; ++e) csr_col[e] = (uint16_t)c->csr_col[e];
     // Channel LLR (Section II-B, step 1) in double, rounded once to float.
     for (int i = 0; i < N; ++i) lch[i] = (float)std::log((1.0 - priors[i]) / priors[i]);
+    // First iteration's C2V magnitudes: every V2C message is a channel LLR then.
+    std::vector<float> c2v0((size_t)N * vstride, 0.f);
+    const float alpha1 = p.alpha > 0.f ? p.alpha : 0.5f;
+    for (int i = 0; i < N; ++i)
+        for (int k = 0; k < (int)cols[i].size(); ++k) {
+            float m = HUGE_VALF;
+            for (int v : rows[cols[i][k].first])
+                if (v != i) m = std::min(m, lch[v]);
+            c2v0[(size_t)i * vstride + k] = std::min(alpha1 * m, 0x1p100f);
+        }
     cudaGetDevice(&c->device);
     cudaDeviceProp prop;
     cudaError_t e = cudaGetDeviceProperties(&prop, c->device);
@@ -578,12 +639,12 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     }
 
     // One allocation for all code arrays.
-    const void *srcs[8] = {row_deg.data(), vchk.data(), lch.data(), row_ptr.data(), csr_col.data(),
-                           masks.data(), layer_ptr.data(), layer_rows.data()};
-    const size_t sizes[8] = {(size_t)M, 2 * vchk.size(), 4 * (size_t)N, 2 * (size_t)(M + 1), 2 * (size_t)nnz,
-                             8 * masks.size(), 2 * layer_ptr.size(), 2 * layer_rows.size()};
-    size_t off[8], sz = 0;
-    for (int k = 0; k < 8; ++k) {
+    const void *srcs[9] = {row_deg.data(), vchk.data(),      lch.data(),        row_ptr.data(), csr_col.data(),
+                           masks.data(),   layer_ptr.data(), layer_rows.data(), c2v0.data()};
+    const size_t sizes[9] = {(size_t)M, 2 * vchk.size(), 4 * (size_t)N, 2 * (size_t)(M + 1), 2 * (size_t)nnz,
+                             8 * masks.size(), 2 * layer_ptr.size(), 2 * layer_rows.size(), 4 * c2v0.size()};
+    size_t off[9], sz = 0;
+    for (int k = 0; k < 9; ++k) {
         off[k] = sz;
         sz += align16(sizes[k]);
     }
@@ -593,7 +654,7 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
         return bpsf_fail(BPSF_ENOMEM, "cudaMalloc(code): %s", cudaGetErrorString(e));
     }
     std::vector<unsigned char> hbuf(sz, 0);
-    for (int k = 0; k < 8; ++k) std::memcpy(hbuf.data() + off[k], srcs[k], sizes[k]);
+    for (int k = 0; k < 9; ++k) std::memcpy(hbuf.data() + off[k], srcs[k], sizes[k]);
     e = cudaMemcpy(c->d_code, hbuf.data(), sz, cudaMemcpyHostToDevice);
     unsigned char *base = (unsigned char *)c->d_code;
     CodeDev &cd = c->code;
@@ -624,6 +685,7 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     cd.n_layers = n_layers;
     cd.layer_ptr = (const uint16_t *)(base + off[6]);
     cd.layer_rows = (const uint16_t *)(base + off[7]);
+    cd.c2v0 = (const float *)(base + off[8]);
     c->default_n_trials = c->n_trials;
     // The per-slot-count layouts: one allocation.
     {
@@ -668,6 +730,13 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     c->tune = default_tuning(c);
     bpsf_tuning cached;
     if (bpsf_tuning_cache_lookup(c, &cached)) c->tune = cached;
+    // Load the column path's kernel and remember its occupancy now, so that a
+    // later call can be recorded into a CUDA graph.
+    for (long long n : {1ll, 1000ll}) {
+        bpsf_plan pl;
+        bpsf_ctx *cs[1] = {c};
+        bpsf_make_plan(cs, 1, &c->tune, false, &pl, false, &n);
+    }
     *out = c;
     return BPSF_OK;
 }
@@ -791,18 +860,21 @@ static bpsf_status decode_impl(bpsf_ctx *c, int64_t n, const uint32_t *synd, int
     cudaSetDevice(c->device);
     bpsf_plan pl;
     bpsf_ctx *cs1[1] = {c};
-    st = bpsf_make_plan(cs1, 1, &c->tune, dbg != nullptr, &pl);
+    const long long shots1[1] = {n};
+    st = bpsf_make_plan(cs1, 1, &c->tune, dbg != nullptr, &pl, false, shots1);
     if (st != BPSF_OK) return st;
     // Shards (the debug dump indexes its arrays by shot, so it keeps one).
     const int K = dbg ? 1 : bpsf_batch_shards(c, n, 1);
     if (K > 1) {
         bpsf_ctx *ck[kMaxShards];
         bpsf_tuning tk[kMaxShards];
+        long long nk[kMaxShards];
         for (int j = 0; j < K; ++j) {
             ck[j] = c;
             tk[j] = c->tune;
+            nk[j] = n * (j + 1) / K - n * j / K;
         }
-        st = bpsf_make_plan(ck, K, tk, false, &pl);
+        st = bpsf_make_plan(ck, K, tk, false, &pl, false, nk);
         if (st != BPSF_OK) return st;
     }
     long long cap_s = 0;
@@ -934,10 +1006,11 @@ extern "C" bpsf_status bpsf_decode_plain(bpsf_ctx *c, int64_t n, const uint32_t 
     // Launch A: one block, one team, one slot, the initial run of one shot.
     bpsf_plan plA, plB;
     bpsf_tuning tA{c->tune.warps_per_team, 1, c->tune.warps_per_team, 0, 1};
-    st = bpsf_make_plan(cs1, 1, &tA, false, &plA);
+    const long long one_shot[1] = {1};
+    st = bpsf_make_plan(cs1, 1, &tA, false, &plA, false, one_shot);
     if (st != BPSF_OK) return st;
     // Launch B: the shot's trials spread over blocks of the tuned shape.
-    st = bpsf_make_plan(cs1, 1, &c->tune, false, &plB);
+    st = bpsf_make_plan(cs1, 1, &c->tune, false, &plB, false, one_shot);
     if (st != BPSF_OK) return st;
     const int trials = std::max(c->n_trials, 1);
     const int per_block = plB.teams_code[0] * plB.S_code[0];
@@ -1133,16 +1206,18 @@ extern "C" bpsf_status bpsf_decode_multi(int32_t n_jobs, const bpsf_job *jobs, v
     std::vector<int> shards(n_jobs);
     std::vector<bpsf_ctx *> scodes;
     std::vector<bpsf_tuning> tunes;
+    std::vector<long long> shots;
     for (int k = 0; k < n_jobs; ++k) {
         shards[k] = bpsf_batch_shards(codes[k], std::max<int64_t>(jobs[k].n_shots, 1), n_jobs);
         for (int q = 0; q < shards[k]; ++q) {
             scodes.push_back(codes[k]);
             tunes.push_back(codes[k]->tune);
+            shots.push_back(jobs[k].n_shots * (q + 1) / shards[k] - jobs[k].n_shots * q / shards[k]);
         }
     }
     const int n_streams = (int)scodes.size();
     bpsf_plan pl;
-    bpsf_status st = bpsf_make_plan(scodes.data(), n_streams, tunes.data(), false, &pl, true);
+    bpsf_status st = bpsf_make_plan(scodes.data(), n_streams, tunes.data(), false, &pl, true, shots.data());
     if (st != BPSF_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<StreamDev> sds(n_streams);
@@ -1243,6 +1318,7 @@ extern "C" bpsf_status bpsf_autotune(bpsf_ctx *c, double p_sample, int64_t n_sam
     float best_ms = 1e30f;
     bpsf_status st = BPSF_OK;
     bpsf_ctx *cs1[1] = {c};
+    c->team_only = true;  // the shapes apply to the team path
     // Time one shape: the best of two decodes after a warm-up decode.
     auto time_shape = [&](const bpsf_tuning &t) -> float {
         c->tune = t;
@@ -1291,6 +1367,7 @@ extern "C" bpsf_status bpsf_autotune(bpsf_ctx *c, double p_sample, int64_t n_sam
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaFree(buf);
+    c->team_only = false;
     c->tune = (st == BPSF_OK) ? best : saved;
     if (st != BPSF_OK) return st;
     {

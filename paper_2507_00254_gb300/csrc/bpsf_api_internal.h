@@ -41,6 +41,7 @@ struct bpsf_ctx {
     void *d_host_stage = nullptr;           // device buffers of bpsf_decode_host
     size_t host_stage_bytes = 0;
     bpsf_tuning tune{};
+    bool team_only = false;                 // not on the column path (while the autotuner times shapes)
     bpsf_work last{};
     long long last_launch_n = 0;
     int last_shards = 1;                    // shards of the last launch (counter blocks bpsf_sync adds up)
@@ -135,9 +136,10 @@ bpsf_status bpsf_ensure_workspace(bpsf_ctx *c, long long n);
 bpsf_status bpsf_ensure_kernel_attrs(int variant, int smem_optin);
 // Plan one launch over n_codes codes; tunes[k] is code k's team shape (a
 // single tuning for a one-code launch).  With shrink, a code whose block does
-// not fit gets fewer slots per team, then fewer teams.
+// not fit gets fewer slots per team, then fewer teams.  shots: the shots of
+// each code in a batch launch (the column path serves small ones), or null.
 bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, bool debug,
-                           bpsf_plan *out, bool shrink = false);
+                           bpsf_plan *out, bool shrink = false, const long long *shots = nullptr);
 void bpsf_launch_plan(const bpsf_plan &pl, bool debug, bpsf::StreamDev *sds, int n, int grid, void *stream);
 bool bpsf_tuning_cache_lookup(const bpsf_ctx *c, bpsf_tuning *out);
 bpsf::StreamDev bpsf_make_stream(const bpsf_ctx *c, const bpsf::JobDev &job, const bpsf::DebugDev *dbg,

@@ -11,6 +11,8 @@ constexpr int kMaxTrials = 4096;  // trials per failed shot
 constexpr int kMaxSlots = 32;     // work items per team
 constexpr int kMaxStreams = 16;   // codes per launch
 constexpr int kMaxComputeWarps = 15;  // plus one manager warp: <= 512 threads per block
+constexpr int kMaxColumnWarps = 19;   // column path: with the manager 20 warps, 96 registers a thread
+constexpr int kColumnThreads = 32 * (kMaxColumnWarps + 1);
 constexpr int kMaxNamedTeams = 15;    // named barriers 1..15 for multi-warp teams
 constexpr int kDVP = 4;           // column entries stored per variable for dv <= 4 codes
 
@@ -57,6 +59,7 @@ struct CodeDev {
     const uint16_t *vpos;        // N x vstride, message positions (0xffff padding), active layout
     const uint16_t *vchk;        // N x vstride, check indices
     const float *lch;            // N, channel LLRs (FP32)
+    const float *c2v0;           // N x vstride, magnitude of the first iteration's C2V messages
     const float *lch_pos;        // P, channel LLR of the variable at each position, active layout
     const uint16_t *row_ptr;     // M+1, CSR (syndrome kernel)
     const uint16_t *csr_col;     // nnz
@@ -188,9 +191,13 @@ struct LayoutOffsets {
     int row_deg, vpos, lch, lch_pos, total;
 };
 
-__host__ __device__ inline LayoutOffsets layout_offsets(int M, int N, int vstride, int P) {
+__host__ __device__ inline LayoutOffsets layout_offsets(int M, int N, int vstride, int P, bool cols = false) {
     LayoutOffsets o;
     int p = 0;
+    if (cols) {  // the column path keeps its tables in registers
+        o.row_deg = o.vpos = o.lch = o.lch_pos = o.total = 0;
+        return o;
+    }
     o.row_deg = p;  p = align_up(p + M, 16);
     o.vpos = p;     p = align_up(p + 2 * N * vstride, 16);
     o.lch = p;      p = align_up(p + 4 * N, 16);
@@ -252,6 +259,7 @@ struct TeamCtl {
     unsigned idle_ns, idle_looks;    //   its current sleep and the looks that found nothing
     unsigned long long iters;  // iterations run by this team (all slots)
     unsigned long long cap;    // team iterations with a running slot, times S
+    int flushed;               // column path: team iterations already in cap
 };
 static_assert(sizeof(TeamCtl) <= 64, "team control block fits its 64 bytes");
 
@@ -290,15 +298,21 @@ struct TeamOffsets {
     int ctl, state, syn, mism, ebits, flips, m, outbox, inflag, inbox, ibstride, post, total;
 };
 
-__host__ __device__ inline TeamOffsets team_offsets(int S, int M, int N, int P, int Ws, int layered, int fb = 2) {
+// Column path: the block's copies of its stream's descriptor and team offsets.
+constexpr int kStreamBytes = (int)((sizeof(StreamDev) + 15) / 16 * 16);
+constexpr int kDescriptorBytes = kStreamBytes + 64;
+static_assert(sizeof(TeamOffsets) <= 64, "team offsets fit their copy");
+
+__host__ __device__ inline TeamOffsets team_offsets(int S, int M, int N, int P, int Ws, int layered, int fb = 2,
+                                                    bool cols = false) {
     TeamOffsets o;
     const int sw = (S * M + 31) / 32;
     int p = 0;
     o.ctl = p;     p += 64;
     o.state = p;   p += (int)sizeof(SlotState) * S;
     o.outbox = p;  p += (int)sizeof(OutBox) * S;
-    o.syn = p;     p += 4 * sw;
-    o.mism = p;    p += 4 * sw;
+    o.syn = p;     p += cols ? align_up(4 * S * Ws, 16) : 4 * sw;
+    o.mism = p;    p += cols ? align_up(4 * M, 16) : 4 * sw;
     o.ebits = p;   p += 4 * S * ((N + 31) / 32);
     o.inflag = p;  p = align_up(p + 4 * S, 16);
     o.ibstride = qentry_bytes(Ws);
@@ -311,9 +325,9 @@ __host__ __device__ inline TeamOffsets team_offsets(int S, int M, int N, int P, 
 }
 
 __host__ __device__ inline int block_smem_bytes(int M, int N, int P, int Ws, int vstride, int S, int teams, int Q,
-                                                int layered, int fb = 2) {
-    return kBlockHeaderBytes + layout_offsets(M, N, vstride, P).total + Q * qentry_bytes(Ws) +
-           teams * team_offsets(S, M, N, P, Ws, layered, fb).total;
+                                                int layered, int fb = 2, bool cols = false) {
+    return kBlockHeaderBytes + (cols ? kDescriptorBytes : 0) + layout_offsets(M, N, vstride, P, cols).total + Q * qentry_bytes(Ws) +
+           teams * team_offsets(S, M, N, P, Ws, layered, fb, cols).total;
 }
 
 // Arguments of one persistent launch: the streams (codes) it serves, by value.
@@ -329,6 +343,7 @@ int kernel_variant(int dc_max, int dv_max);  // smallest variant that fits, -1 i
 int kernel_variant_dv(int variant);          // column table width of a variant
 int kernel_variant_full_regs(int variant);   // its one-block, full-register instance
 int kernel_variant_byte_flips(int variant);  // its one-block instance with one-byte flip words, -1 if none
+int kernel_variant_columns(int variant, int fb);  // its column-path instance, -1 if none
 int kernel_variant_mixed(int variant);       // its instance with the exact (6, 4, 3) path as well, -1 if none
 const void *persistent_kernel_ptr(int variant, bool debug, bool layered);
 void launch_persistent(int variant, bool debug, bool layered, int grid, int block, int smem, const LaunchArgs &args,

@@ -21,6 +21,8 @@ KernelFn kernel_fn_v4(bool debug, bool lay);
 KernelFn kernel_fn_v5(bool debug, bool lay);
 KernelFn kernel_fn_v6(bool debug, bool lay);
 KernelFn kernel_fn_v7(bool debug, bool lay);
+KernelFn kernel_fn_v8(bool debug, bool lay);
+KernelFn kernel_fn_v9(bool debug, bool lay);
 
 // ---------------------------------------------------------------------------
 // Variants and launch helpers.
@@ -35,7 +37,7 @@ struct Variant {
 // kernel_variant_full_regs, kernel_variant_byte_flips and
 // kernel_variant_mixed).
 static const Variant kVariants[] = {{6, 4, 3}, {6, 4, 0}, {8, 4, 0}, {16, 8, 0}, {32, 16, 0}, {6, 4, 3}, {6, 4, 3},
-                                    {8, 4, 0}};
+                                    {8, 4, 0}, {6, 4, 3}, {6, 4, 3}};
 static const int kNumVariants = 5;
 
 // Smallest variant that fits.  The exact-degree variant serves codes with
@@ -64,7 +66,9 @@ static KernelFn kernel_fn(int variant, bool debug, bool lay) {
         case 4: return kernel_fn_v4(debug, lay);
         case 5: return kernel_fn_v5(debug, lay);
         case 6: return kernel_fn_v6(debug, lay);
-        default: return kernel_fn_v7(debug, lay);
+        case 7: return kernel_fn_v7(debug, lay);
+        case 8: return kernel_fn_v8(debug, lay);
+        default: return kernel_fn_v9(debug, lay);
     }
 }
 
@@ -75,6 +79,9 @@ int kernel_variant_full_regs(int variant) { return variant == 0 ? 5 : variant; }
 
 // The instance with one-byte flip words (full registers, no layered path), or -1.
 int kernel_variant_byte_flips(int variant) { return (variant == 0 || variant == 5) ? 6 : -1; }
+
+// The column-path instance of a variant for fb-byte flip words (no layered path), or -1.
+int kernel_variant_columns(int variant, int fb) { return variant == 0 ? (fb == 1 ? 9 : 8) : -1; }
 
 // The instance that runs variant 2's codes together with exact (6, 4, 3)
 // codes on their own path, or -1.

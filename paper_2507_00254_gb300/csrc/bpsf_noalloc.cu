@@ -91,7 +91,8 @@ extern "C" bpsf_status bpsf_decode_noalloc(bpsf_ctx *c, int64_t n, const uint32_
     if (st != BPSF_OK) return st;
     bpsf_plan pl;
     bpsf_ctx *cs1[1] = {c};
-    st = bpsf_make_plan(cs1, 1, &c->tune, false, &pl);
+    const long long shots[1] = {n};
+    st = bpsf_make_plan(cs1, 1, &c->tune, false, &pl, false, shots);
     if (st != BPSF_OK) return st;
     // Carve the counters and the record ring out of the array.
     const long long ring = bpsf_record_ring(n);

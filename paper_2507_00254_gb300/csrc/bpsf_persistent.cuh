@@ -58,6 +58,14 @@ namespace bpsf {
 
 #define FULLMASK 0xffffffffu
 
+// Keeps a loop-invariant value in its register.  The descriptors sit in
+// parameter space, indexed by the stream; left alone, the compiler loads such
+// values again in every iteration (about 120 cycles for each load).
+__device__ __forceinline__ int keep(int x) {
+    asm volatile("" : "+r"(x));
+    return x;
+}
+
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -104,7 +112,8 @@ struct BlockHdr {
     int stream, cmd;
     volatile int exit;            // manager -> teams: leave the team loop
     volatile unsigned heartbeat;  // manager passes; idle teams give up only if it stalls
-    int pad[12];
+    unsigned long long wait_ns;   // bound on any device-side wait (column path)
+    int pad[10];
 };
 
 struct LayoutMem {
@@ -616,13 +625,99 @@ __device__ __forceinline__ void layered_iteration(const StreamDev &sd, const Lay
 // without a round trip through the manager.
 // ---------------------------------------------------------------------------
 
+// The record of slot s's failed initial run: Phi = top(flip_count, w) (keys
+// (count << 16 | 0xffff - i) are distinct, so each round takes the largest
+// key below the previous one: count descending, index ascending), the shot's
+// syndrome, an empty selection and the provisional output (the initial run's
+// e, not converged); only then is the record published for the trials.
+// Called by one warp, with the slot's flip words and packed decision in place.
+template <bool DEBUG, int FB, bool COLS>
+__device__ __forceinline__ void publish_failure(const StreamDev &sd, const TeamMem &T, int lgS, int s, int lane,
+                                                unsigned long long wait_ns) {
+    const CodeDev &cd = sd.code;
+    const int N = cd.N, Wn = cd.Wn;
+    const JobDev &job = sd.job;
+    const long long shot = T.st[s].shot;
+    const long long row = (sd.flags & kServe) ? (shot % sd.serve.rows) : shot;
+    // Phi into lane registers: lane r % 32 holds Phi[r] (r < 32 in phi0, else phi1).
+    int phi0 = -1, phi1 = -1;
+    unsigned thr = 0xffffffffu;
+    for (int r = 0; r < cd.w; ++r) {
+        unsigned best = 0;
+        for (int i = lane; i < N; i += 32) {
+            const unsigned key =
+                (flip_count<FB>((unsigned)flipw<FB>(T)[(i << lgS) + s]) << 16) | (0xffffu - (unsigned)i);
+            if (key < thr && key > best) best = key;
+        }
+        best = __reduce_max_sync(FULLMASK, best);
+        const int phi_r = (int)(0xffffu - (best & 0xffffu));
+        if (lane == (r & 31)) {
+            if (r < 32)
+                phi0 = phi_r;
+            else
+                phi1 = phi_r;
+        }
+        if (DEBUG && lane == 0 && sd.dbg.phi) sd.dbg.phi[shot * cd.w + r] = phi_r;
+        thr = best;
+    }
+    // The next failure number and its record, once free (a bounded wait;
+    // more failed shots in flight than records is reported).
+    unsigned long long q = 0;
+    if (lane == 0) {
+        q = atomicAdd(&sd.ctr->rec_count, 1ull);
+        const unsigned long long *qs = sd.rec.qseq + (q & (unsigned long long)(sd.rec.cap - 1));
+        auto busy = [&] {
+            const unsigned long long v = ld_acquire_u64(qs);
+            return v != 0ull && !(v & kRecFree);
+        };
+        if (busy()) {
+            const unsigned long long t0 = globaltimer_ns();
+            while (busy()) {
+                if (globaltimer_ns() - t0 > wait_ns) {
+                    atomicOr(&sd.ctr->status, kDevRecordOverflow);
+                    break;
+                }
+                __nanosleep(256);
+            }
+        }
+    }
+    q = __shfl_sync(FULLMASK, q, 0);
+    const long long rs = (long long)(q & (unsigned long long)(sd.rec.cap - 1));
+    if (lane < cd.w) sd.rec.phi[rs * cd.w + lane] = phi0;
+    if (lane + 32 < cd.w) sd.rec.phi[rs * cd.w + lane + 32] = phi1;
+    // The slot's syndrome: its own words (COLS), or bit j*S + s of the team's words for check j.
+    if (COLS) {
+        for (int w = lane; w < cd.Ws; w += 32) sd.rec.synd[rs * cd.Ws + w] = T.syn[s * cd.Ws + w];
+    } else {
+        for (int w = 0; w < cd.Ws; ++w) {
+            const int j = 32 * w + lane;
+            const int b = (j << lgS) + s;
+            const unsigned bit = j < cd.M ? (T.syn[b >> 5] >> (b & 31)) & 1u : 0u;
+            const unsigned word = __ballot_sync(FULLMASK, bit != 0u);
+            if (lane == 0) sd.rec.synd[rs * cd.Ws + w] = word;
+        }
+    }
+    __syncwarp();  // lane 0's decision words are visible to the warp
+    uint32_t *out = job.corr + row * job.corr_stride;
+    for (int w = lane; w < Wn; w += 32) {
+        sd.rec.win[rs * Wn + w] = ~0ull;
+        out[w] = T.ebits[s * Wn + w];
+    }
+    if (lane == 0) {
+        job.conv[row] = 0;
+        job.iters[row] = (int16_t)cd.max_iter;
+        if (job.stage) job.stage[row] = 2;
+        sd.rec.done[rs] = 0u;
+        sd.rec.best[rs] = ~0ull;
+        sd.rec.qshot[rs] = shot;
+    }
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) st_release_u64(sd.rec.qseq + rs, q + 1ull);
+}
+
 // Pack finished slot s into its outbox: the hard decision into words and the
-// run's facts.  A failed initial run (with trials) also gets its record
-// here: Phi = top(flip_count, w) (keys (count << 16 | 0xffff - i) are
-// distinct, so each round takes the largest key below the previous one:
-// count descending, index ascending), the shot's syndrome, an empty
-// selection and the provisional output (the initial run's e, not
-// converged), and only then is the record published for the trials.
+// run's facts.  A failed initial run (with trials) also gets its record here.
 template <bool DEBUG, int FB>
 __device__ __forceinline__ void team_pack(const StreamDev &sd, const TeamMem &T, int lgS, int s, int lane,
                                           unsigned long long wait_ns) {
@@ -637,82 +732,7 @@ __device__ __forceinline__ void team_pack(const StreamDev &sd, const TeamMem &T,
         if (lane == 0) T.ebits[s * Wn + w] = word;
     }
     const int kind = ss->kind, outcome = ss->outcome;
-    if (kind == 1 && outcome == 2 && cd.w > 0) {
-        const JobDev &job = sd.job;
-        const long long shot = ss->shot;
-        const long long row = (sd.flags & kServe) ? (shot % sd.serve.rows) : shot;
-        // Phi into lane registers: lane r % 32 holds Phi[r] (r < 32 in phi0, else phi1).
-        int phi0 = -1, phi1 = -1;
-        unsigned thr = 0xffffffffu;
-        for (int r = 0; r < cd.w; ++r) {
-            unsigned best = 0;
-            for (int i = lane; i < N; i += 32) {
-                const unsigned key =
-                    (flip_count<FB>((unsigned)flipw<FB>(T)[(i << lgS) + s]) << 16) | (0xffffu - (unsigned)i);
-                if (key < thr && key > best) best = key;
-            }
-            best = __reduce_max_sync(FULLMASK, best);
-            const int phi_r = (int)(0xffffu - (best & 0xffffu));
-            if (lane == (r & 31)) {
-                if (r < 32)
-                    phi0 = phi_r;
-                else
-                    phi1 = phi_r;
-            }
-            if (DEBUG && lane == 0 && sd.dbg.phi) sd.dbg.phi[shot * cd.w + r] = phi_r;
-            thr = best;
-        }
-        // The next failure number and its record, once free (a bounded wait;
-        // more failed shots in flight than records is reported).
-        unsigned long long q = 0;
-        if (lane == 0) {
-            q = atomicAdd(&sd.ctr->rec_count, 1ull);
-            const unsigned long long *qs = sd.rec.qseq + (q & (unsigned long long)(sd.rec.cap - 1));
-            auto busy = [&] {
-                const unsigned long long v = ld_acquire_u64(qs);
-                return v != 0ull && !(v & kRecFree);
-            };
-            if (busy()) {
-                const unsigned long long t0 = globaltimer_ns();
-                while (busy()) {
-                    if (globaltimer_ns() - t0 > wait_ns) {
-                        atomicOr(&sd.ctr->status, kDevRecordOverflow);
-                        break;
-                    }
-                    __nanosleep(256);
-                }
-            }
-        }
-        q = __shfl_sync(FULLMASK, q, 0);
-        const long long rs = (long long)(q & (unsigned long long)(sd.rec.cap - 1));
-        if (lane < cd.w) sd.rec.phi[rs * cd.w + lane] = phi0;
-        if (lane + 32 < cd.w) sd.rec.phi[rs * cd.w + lane + 32] = phi1;
-        // The slot's syndrome (check j sits at bit j*S + s of the team's words).
-        for (int w = 0; w < cd.Ws; ++w) {
-            const int j = 32 * w + lane;
-            const int b = (j << lgS) + s;
-            const unsigned bit = j < cd.M ? (T.syn[b >> 5] >> (b & 31)) & 1u : 0u;
-            const unsigned word = __ballot_sync(FULLMASK, bit != 0u);
-            if (lane == 0) sd.rec.synd[rs * cd.Ws + w] = word;
-        }
-        __syncwarp();  // lane 0's decision words are visible to the warp
-        uint32_t *out = job.corr + row * job.corr_stride;
-        for (int w = lane; w < Wn; w += 32) {
-            sd.rec.win[rs * Wn + w] = ~0ull;
-            out[w] = T.ebits[s * Wn + w];
-        }
-        if (lane == 0) {
-            job.conv[row] = 0;
-            job.iters[row] = (int16_t)cd.max_iter;
-            if (job.stage) job.stage[row] = 2;
-            sd.rec.done[rs] = 0u;
-            sd.rec.best[rs] = ~0ull;
-            sd.rec.qshot[rs] = shot;
-        }
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) st_release_u64(sd.rec.qseq + rs, q + 1ull);
-    }
+    if (kind == 1 && outcome == 2 && cd.w > 0) publish_failure<DEBUG, FB, false>(sd, T, lgS, s, lane, wait_ns);
     if (DEBUG && kind == 1 && sd.dbg.flips)
         for (int i = lane; i < N; i += 32)
             sd.dbg.flips[ss->shot * N + i] = (uint16_t)flip_count<FB>((unsigned)flipw<FB>(T)[(i << lgS) + s]);
@@ -1013,6 +1033,12 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
         svc = run == 0u || (since >= chunk && run != full);
     }
 }
+
+}  // namespace bpsf
+
+#include "bpsf_columns.cuh"
+
+namespace bpsf {
 
 // ---------------------------------------------------------------------------
 // Manager warp.
@@ -1521,8 +1547,8 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
 // for codes with exactly six ones per row and three per column, so such codes
 // keep their specialised path in a launch that mixes them with codes of
 // wider rows (the layouts agree: both have column tables of width DVS).
-template <int DC, int DVS, int DVX, bool DEBUG, int MINB, bool LAY, int FB = 2, bool MIX = false>
-__global__ void __launch_bounds__(512, MINB) bpsf_persistent(const __grid_constant__ KernelParams kp) {
+template <int DC, int DVS, int DVX, bool DEBUG, int MINB, bool LAY, int FB = 2, bool MIX = false, bool COLS = false>
+__global__ void __launch_bounds__(COLS ? kColumnThreads : 512, MINB) bpsf_persistent(const __grid_constant__ KernelParams kp) {
     extern __shared__ __align__(16) unsigned char smem[];
     BlockHdr *hdr = reinterpret_cast<BlockHdr *>(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1610,12 +1636,23 @@ __global__ void __launch_bounds__(512, MINB) bpsf_persistent(const __grid_consta
             continue;
         }
         waiting = false;
-        const StreamDev &sd = kp.streams[sid];
+        if (COLS && sid != cur) {
+            // The column path reads its descriptor in shared memory.
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(&kp.streams[sid]);
+            for (int k = tid; k < (int)(sizeof(StreamDev) / 4); k += blockDim.x)
+                reinterpret_cast<uint32_t *>(smem + kBlockHeaderBytes)[k] = src[k];
+            const StreamDev &d = kp.streams[sid];
+            if (tid == 0)
+                *reinterpret_cast<TeamOffsets *>(smem + kBlockHeaderBytes + kStreamBytes) =
+                    team_offsets(d.S, d.code.M, d.code.N, d.code.P, d.code.Ws, 0, FB, true);
+            __syncthreads();
+        }
+        const StreamDev &sd = COLS ? *reinterpret_cast<const StreamDev *>(smem + kBlockHeaderBytes) : kp.streams[sid];
         const CodeDev &cd = sd.code;
         const int S = sd.S, W = sd.W, teams = sd.teams;
-        const LayoutOffsets lo = layout_offsets(cd.M, cd.N, DVS, cd.P);
-        unsigned char *lay = smem + kBlockHeaderBytes;
-        if (sid != cur) {
+        const LayoutOffsets lo = layout_offsets(cd.M, cd.N, DVS, cd.P, COLS);
+        unsigned char *lay = smem + kBlockHeaderBytes + (COLS ? kDescriptorBytes : 0);
+        if (sid != cur && !COLS) {
             uint8_t *rd = lay + lo.row_deg;
             uint16_t *vp = reinterpret_cast<uint16_t *>(lay + lo.vpos);
             float *lc = reinterpret_cast<float *>(lay + lo.lch);
@@ -1624,10 +1661,13 @@ __global__ void __launch_bounds__(512, MINB) bpsf_persistent(const __grid_consta
             for (int k = tid; k < cd.N * DVS; k += blockDim.x) vp[k] = cd.vpos[k];
             for (int k = tid; k < cd.N; k += blockDim.x) lc[k] = cd.lch[k];
             for (int k = tid; k < cd.P; k += blockDim.x) lp[k] = cd.lch_pos[k];
-            cur = sid;
         }
+        cur = sid;
         // Every slot starts empty; teams start idle.
-        const TeamOffsets to = team_offsets(S, cd.M, cd.N, cd.P, cd.Ws, cd.layered, FB);
+        TeamOffsets to_reg;
+        if (!COLS) to_reg = team_offsets(S, cd.M, cd.N, cd.P, cd.Ws, cd.layered, FB);
+        const TeamOffsets &to =
+            COLS ? *reinterpret_cast<const TeamOffsets *>(smem + kBlockHeaderBytes + kStreamBytes) : to_reg;
         unsigned char *qbase = lay + lo.total;
         unsigned char *team_base = qbase + Q * qentry_bytes(cd.Ws);
         for (int k = tid; k < teams * S; k += blockDim.x) {
@@ -1649,15 +1689,16 @@ __global__ void __launch_bounds__(512, MINB) bpsf_persistent(const __grid_consta
         // only their own slot's bits, and the padding bits past S*M are read
         // by the convergence test.
         {
-            const int sw = (to.mism - to.syn) / 4;
-            for (int k = tid; k < teams * 2 * sw; k += blockDim.x) {
-                const int t = k / (2 * sw), w = k - t * 2 * sw;
+            const int sw = (to.ebits - to.syn) / 4;
+            for (int k = tid; k < teams * sw; k += blockDim.x) {
+                const int t = k / sw, w = k - t * sw;
                 reinterpret_cast<uint32_t *>(team_base + t * to.total + to.syn)[w] = 0u;
             }
         }
         if (tid == 0) {
             hdr->exit = 0;
             hdr->heartbeat = 0u;
+            hdr->wait_ns = kp.wait_ns;
         }
         __syncthreads();
         LayoutMem L;
@@ -1672,7 +1713,13 @@ __global__ void __launch_bounds__(512, MINB) bpsf_persistent(const __grid_consta
             if (team < teams) {
                 TeamMem T = team_mem(team_base + team * to.total, to);
                 const int ttid = tid - 32 - team * W * 32;
-                if (MIX && cd.regular && cd.DC == 6 && cd.dv_max == 3)
+                if constexpr (COLS) {
+                    const int tb = keep((int)(team_base - smem) + team * to.total);
+                    if (S == 4)
+                        column_loop<DC, DVX, DVS, 4, DEBUG, FB>(sd, to, hdr, tb, W, ttid, 1 + team);
+                    else
+                        column_loop<DC, DVX, DVS, 1, DEBUG, FB>(sd, to, hdr, tb, W, ttid, 1 + team);
+                } else if (MIX && cd.regular && cd.DC == 6 && cd.dv_max == 3)
                     team_loop<6, DVS, 3, DEBUG, MINB, LAY, FB>(sd, L, T, hdr, S, W, ttid, 1 + team, kp.wait_ns);
                 else
                     team_loop<DC, DVS, DVX, DEBUG, MINB, LAY, FB>(sd, L, T, hdr, S, W, ttid, 1 + team, kp.wait_ns);

@@ -11,7 +11,7 @@ torch = pytest.importorskip("torch")
 import oracle  # noqa: E402
 from oracle import Code, Params as OParams  # noqa: E402
 from paper_2507_00254_gb300 import bpsf as B  # noqa: E402
-from paper_2507_00254_gb300 import harness  # noqa: E402
+from paper_2507_00254_gb300 import codes, harness  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -56,10 +56,36 @@ def test_irregular_rows_and_columns(dc, dv, slots, layered, alpha):
 @pytest.mark.parametrize("m", [33, 64])
 def test_regular_rows(m, slots, max_iter):
     rng = np.random.default_rng(m + slots)
-    run(rng, regular(rng, m), slots, False, 0.625, max_iter)
+    run(rng, regular(rng, m), slots, False, 0.625, max_iter, blocks=1)
 
 
-def run(rng, h, slots, layered, alpha, max_iter=40):
+# A lane per column: from one warp to the nineteen that a block holds (and one
+# column more, which the teams serve), rows past the 128 of one residual look.
+@pytest.mark.parametrize("m,alpha,max_iter", [(8, 0.625, 40), (16, 0.0, 40), (17, 0.625, 200), (48, 0.0, 200),
+                                              (129, 0.625, 40), (304, 0.625, 30), (305, 0.625, 30)])
+def test_column_path(m, alpha, max_iter):
+    rng = np.random.default_rng(m)
+    run(rng, regular(rng, m), 4, False, alpha, max_iter)
+
+
+@pytest.mark.parametrize("select", [B.BPSF_SELECT_MIN_WEIGHT, B.BPSF_SELECT_FIRST])
+@pytest.mark.parametrize("shots", [1, 7, 8, 500])  # one and four slots per team
+def test_column_path_equals_teams(shots, select):
+    c = codes.bb("bb144")
+    d = B.Decoder(c.ptr, c.idx, c.M, c.N, np.full(c.N, 0.07), B.Params(max_iter=60, w=6, short_iter=20, select=select))
+    rng = np.random.default_rng(shots)
+    e = (rng.random((shots, c.N)) < 0.08).astype(np.uint8)
+    synd = d.syndrome(torch.from_numpy(harness.pack_rows(e).view(np.int32)).cuda())
+    got = d.decode(synd)
+    work = d.last_work()
+    d.tuning = (1, 4, 8, 1, 1)  # blocks per SM given: the teams
+    want = d.decode(synd)
+    assert all(torch.equal(got[k], want[k]) for k in got)
+    if select == B.BPSF_SELECT_MIN_WEIGHT:
+        assert all(work[k] == v for k, v in d.last_work().items() if k != "slot_capacity")
+
+
+def run(rng, h, slots, layered, alpha, max_iter=40, blocks=0):
     m, n = h.shape
     idx = np.concatenate([np.nonzero(r)[0] for r in h])
     ptr = np.concatenate([[0], np.cumsum(h.sum(axis=1))])
@@ -67,7 +93,7 @@ def run(rng, h, slots, layered, alpha, max_iter=40):
     P = B.Params(max_iter=max_iter, alpha=alpha, w=3, short_iter=9, layered=layered)
     d = B.Decoder(ptr, idx, m, n, priors, P)
     for warps in (1, 2):
-        d.tuning = (warps, slots, 4, 0, 1)
+        d.tuning = (warps, slots, 4, blocks, 1)
         shots = 301
         e = (rng.random((shots, n)) < priors).astype(np.uint8)
         s = (e.astype(np.int64) @ h.T.astype(np.int64) & 1).astype(np.uint8)
