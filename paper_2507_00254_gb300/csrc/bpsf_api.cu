@@ -163,24 +163,23 @@ static cudaError_t blocks_per_sm(const void *fn, int block, int smem, int *occ) 
 constexpr long long kColumnShots = 1500000;
 
 static void plan_columns(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, const long long *shots,
-                         int base, bpsf_plan *out, int *variant, int *B, int *smem, long long *grid_max, int Q) {
-    if (kernel_variant_columns(base, 2) < 0) return;
+                         int dc, int dv, bpsf_plan *out, int *variant, int *B, int *smem, long long *grid_max, int Q) {
+    if (kernel_variant_columns(dc, dv, 2) < 0) return;
     long long work = 0;
     int fb = 1;
     for (int k = 0; k < n_codes; ++k) {
         if ((codes[k]->N + 31) / 32 > kMaxColumnWarps || codes[k]->team_only || tunes[k].blocks_per_sm > 0) return;
         if (codes[k]->p.max_iter > 127) fb = 2;
-        if (shots[k] > kColumnShots) return;
-        work += shots[k] * codes[k]->N;
+        work += std::min(shots[k], kColumnShots) * codes[k]->N;
     }
-    if (work > kColumnShots) return;
-    const int vstride = kernel_variant_dv(base);
+    if (dc == 6 && work > kColumnShots) return;
+    const int vstride = codes[0]->vstride;
     int warps = 0, bytes = 0;
     long long blocks = 0;
     for (int k = 0; k < n_codes; ++k) {
         const bpsf_ctx *c = codes[k];
         const int W = (c->N + 31) / 32, teams = std::min(kMaxNamedTeams, kMaxColumnWarps / W);
-        const long long runs = shots[k] * (1 + c->n_trials);
+        const long long runs = std::min(shots[k], kColumnShots) * (1 + c->n_trials);
         const int S = runs <= (long long)teams * c->sm_count ? 1 : 4;
         out->W_code[k] = W;
         out->S_code[k] = S;
@@ -190,7 +189,7 @@ static void plan_columns(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning 
         bytes = std::max(bytes, block_smem_bytes(c->M, c->N, c->code.lay[layout_index(S)].P, c->Ws, vstride, S, teams, Q,
                                                  0, fb, true));
     }
-    *variant = kernel_variant_columns(base, fb);
+    *variant = kernel_variant_columns(dc, dv, fb);
     *B = warps;
     *smem = bytes;
     *grid_max = std::max(1ll, blocks);
@@ -274,7 +273,7 @@ bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tunin
     }
     long long grid_max = 1ll << 30;
     if (shots && all_regular && !layered)
-        plan_columns(codes, n_codes, tunes, shots, kernel_variant(-dc, dv), out, &variant, &B, &smem, &grid_max, Q);
+        plan_columns(codes, n_codes, tunes, shots, dc, dv, out, &variant, &B, &smem, &grid_max, Q);
     bpsf_status st = bpsf_ensure_kernel_attrs(variant, c0->smem_optin);
     if (st != BPSF_OK) return st;
     const int block = 32 * (B + 1);

@@ -23,6 +23,8 @@ KernelFn kernel_fn_v6(bool debug, bool lay);
 KernelFn kernel_fn_v7(bool debug, bool lay);
 KernelFn kernel_fn_v8(bool debug, bool lay);
 KernelFn kernel_fn_v9(bool debug, bool lay);
+KernelFn kernel_fn_v10(bool debug, bool lay);
+KernelFn kernel_fn_v11(bool debug, bool lay);
 
 // ---------------------------------------------------------------------------
 // Variants and launch helpers.
@@ -33,11 +35,12 @@ struct Variant {
 };
 // Index 5 is the full-register instance of variant 0 and index 6 the same
 // with one-byte flip words; index 7 is variant 2 with the exact (6, 4, 3)
-// path for the codes that have it (none is chosen by kernel_variant; see
+// path for the codes that have it and 8 to
+// 11 are the column-path instances (none is chosen by kernel_variant; see
 // kernel_variant_full_regs, kernel_variant_byte_flips and
 // kernel_variant_mixed).
 static const Variant kVariants[] = {{6, 4, 3}, {6, 4, 0}, {8, 4, 0}, {16, 8, 0}, {32, 16, 0}, {6, 4, 3}, {6, 4, 3},
-                                    {8, 4, 0}, {6, 4, 3}, {6, 4, 3}};
+                                    {8, 4, 0}, {6, 4, 3}, {6, 4, 3}, {10, 8, 5}, {10, 8, 5}};
 static const int kNumVariants = 5;
 
 // Smallest variant that fits.  The exact-degree variant serves codes with
@@ -68,7 +71,9 @@ static KernelFn kernel_fn(int variant, bool debug, bool lay) {
         case 6: return kernel_fn_v6(debug, lay);
         case 7: return kernel_fn_v7(debug, lay);
         case 8: return kernel_fn_v8(debug, lay);
-        default: return kernel_fn_v9(debug, lay);
+        case 9: return kernel_fn_v9(debug, lay);
+        case 10: return kernel_fn_v10(debug, lay);
+        default: return kernel_fn_v11(debug, lay);
     }
 }
 
@@ -80,8 +85,13 @@ int kernel_variant_full_regs(int variant) { return variant == 0 ? 5 : variant; }
 // The instance with one-byte flip words (full registers, no layered path), or -1.
 int kernel_variant_byte_flips(int variant) { return (variant == 0 || variant == 5) ? 6 : -1; }
 
-// The column-path instance of a variant for fb-byte flip words (no layered path), or -1.
-int kernel_variant_columns(int variant, int fb) { return variant == 0 ? (fb == 1 ? 9 : 8) : -1; }
+// The column-path instance for codes of exactly dc ones per row and dv per
+// column, fb-byte flip words and no layered schedule, or -1.
+int kernel_variant_columns(int dc, int dv, int fb) {
+    for (int v = 8; v < 12; v += 2)
+        if (kVariants[v].dc == dc && kVariants[v].dvx == dv) return v + (fb == 1 ? 1 : 0);
+    return -1;
+}
 
 // The instance that runs variant 2's codes together with exact (6, 4, 3)
 // codes on their own path, or -1.
