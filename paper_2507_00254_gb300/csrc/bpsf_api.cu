@@ -52,6 +52,10 @@ extern "C" const char *bpsf_status_str(bpsf_status s) {
 // waiting for other blocks to publish trials).
 const unsigned long long kBpsfWaitNs = 5ull * 1000 * 1000 * 1000;
 
+// A context's counter blocks, one for each stream of a launch; in the workspace
+// the record numbers follow, so one memset clears both before a launch.
+static constexpr size_t kCounterBytes = kMaxStreams * sizeof(StreamCounters);
+
 static size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
 // ---------------------------------------------------------------------------
@@ -59,8 +63,16 @@ static size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 // ---------------------------------------------------------------------------
 
 static void free_workspace(bpsf_ctx *c) {
-    if (c->d_rec) cudaFree(c->d_rec);
+    if (c->d_rec) {
+        // The counters of the last launch stay readable (bpsf_sync).
+        if (c->d_ctr_last == c->w_ctr) {
+            cudaMemcpy(c->d_ctr, c->w_ctr, kCounterBytes, cudaMemcpyDeviceToDevice);
+            c->d_ctr_last = c->d_ctr;
+        }
+        cudaFree(c->d_rec);
+    }
     c->d_rec = nullptr;
+    c->w_ctr = nullptr;
     c->rec = Records{};
     c->rec_cap = 0;
 }
@@ -76,7 +88,6 @@ extern "C" void bpsf_destroy(bpsf_ctx *c) {
     if (c->d_layouts) cudaFree(c->d_layouts);
     if (c->d_ctr) cudaFree(c->d_ctr);
     if (c->h_ctr) cudaFreeHost(c->h_ctr);
-    if (c->h_flag) cudaFreeHost(c->h_flag);
     if (c->h_preset) cudaFreeHost(c->h_preset);
     if (c->d_host_stage) cudaFree(c->d_host_stage);
     if (prev >= 0) cudaSetDevice(prev);
@@ -719,7 +730,6 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_ctr, kMaxStreams * sizeof(StreamCounters));
     if (e == cudaSuccess) e = cudaMemset(c->d_ctr, 0, kMaxStreams * sizeof(StreamCounters));
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_ctr, kMaxStreams * sizeof(StreamCounters));
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_flag, 64);
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_preset, sizeof(StreamCounters));
     if (e != cudaSuccess) {
         bpsf_destroy(c);
@@ -767,22 +777,22 @@ bpsf_status bpsf_ensure_workspace_sharded(bpsf_ctx *c, long long n, int shards, 
     *shard_cap = cap_s;
     const long long cap = cap_s * shards;  // a power of two: shards is one
     if (cap <= c->rec_cap) return BPSF_OK;
-    const size_t total = bpsf_records_bytes(cap, c->p.w, c->Ws, c->Wn, 16);
+    const size_t total = kCounterBytes + bpsf_records_bytes(cap, c->p.w, c->Ws, c->Wn, 16);
     free_workspace(c);
     void *mem = nullptr;
     cudaError_t e = cudaMalloc(&mem, total);
     if (e != cudaSuccess) return bpsf_fail(BPSF_ENOMEM, "workspace of %zu bytes: %s", total, cudaGetErrorString(e));
     c->d_rec = mem;
-    c->rec = bpsf_records_carve(mem, cap, c->p.w, c->Ws, c->Wn, 16);
+    c->w_ctr = static_cast<StreamCounters *>(mem);
+    c->rec = bpsf_records_carve(static_cast<unsigned char *>(mem) + kCounterBytes, cap, c->p.w, c->Ws, c->Wn, 16);
     c->rec_cap = cap;
     return BPSF_OK;
 }
 
-// Every record of the ring reads free before a launch.
-static bpsf_status clear_queue(bpsf_ctx *c, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(c->rec.qseq, 0, 8 * (size_t)c->rec.cap, s);
-    if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-    return BPSF_OK;
+// The counters read zero and the first n records free before a launch (one
+// memset: two cost a small call about 4 us).
+static cudaError_t clear_workspace(bpsf_ctx *c, long long n, cudaStream_t s) {
+    return cudaMemsetAsync(c->w_ctr, 0, kCounterBytes + 8 * (size_t)n, s);
 }
 
 void bpsf_shard_streams(const bpsf_ctx *c, const JobDev &job, int shards, long long shard_cap, const DebugDev *dbg,
@@ -799,7 +809,7 @@ void bpsf_shard_streams(const bpsf_ctx *c, const JobDev &job, int shards, long l
         jj.stage = job.stage ? job.stage + a : nullptr;
         jj.n_shots = b - a;
         StreamDev sd = bpsf_make_stream(c, jj, dbg, 0);
-        sd.ctr = c->d_ctr + j;
+        sd.ctr = c->w_ctr + j;
         const long long r0 = (long long)j * shard_cap;
         Records &r = sd.rec;
         r.qseq = c->rec.qseq + r0;
@@ -880,17 +890,16 @@ static bpsf_status decode_impl(bpsf_ctx *c, int64_t n, const uint32_t *synd, int
     st = bpsf_ensure_workspace_sharded(c, n, K, &cap_s);
     if (st != BPSF_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(c->d_ctr, 0, K * sizeof(StreamCounters), s);
+    cudaError_t e = clear_workspace(c, c->rec.cap, s);
     if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-    st = clear_queue(c, s);
-    if (st != BPSF_OK) return st;
     JobDev job{synd, corr, conv, iters, stage, n, ss, cs};
     StreamDev sds[kMaxShards];
     bpsf_shard_streams(c, job, K, cap_s, dbg, sds);
     bpsf_launch_plan(pl, dbg != nullptr, sds, K, pl.grid, stream);
     e = cudaGetLastError();
     if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "kernel launch: %s", cudaGetErrorString(e));
-    c->d_ctr_last = c->d_ctr;
+    c->d_ctr_last = c->w_ctr;
+    c->last_stream = stream;
     c->last_shards = K;
     c->last_launch_n = n;
     return BPSF_OK;
@@ -911,12 +920,18 @@ extern "C" bpsf_status bpsf_decode_debug(bpsf_ctx *c, int64_t n, const uint32_t 
 
 extern "C" bpsf_status bpsf_sync(bpsf_ctx *c, void *stream) {
     if (!c) return bpsf_fail(BPSF_EINVAL, "ctx is NULL");
-    cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
-    if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "cudaStreamSynchronize: %s", cudaGetErrorString(e));
     StreamCounters *dc = c->d_ctr_last ? c->d_ctr_last : c->d_ctr;
     const int K = std::max(1, c->last_shards);
-    e = cudaMemcpy(c->h_ctr, dc, K * sizeof(StreamCounters), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "cudaMemcpy: %s", cudaGetErrorString(e));
+    cudaError_t e = cudaSuccess;
+    if (stream == c->last_stream) {
+        // The counters come with the stream's own work: one wait.
+        e = cudaMemcpyAsync(c->h_ctr, dc, K * sizeof(StreamCounters), cudaMemcpyDeviceToHost, (cudaStream_t)stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);
+    } else {
+        e = cudaStreamSynchronize((cudaStream_t)stream);
+        if (e == cudaSuccess) e = cudaMemcpy(c->h_ctr, dc, K * sizeof(StreamCounters), cudaMemcpyDeviceToHost);
+    }
+    if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "waiting for the stream: %s", cudaGetErrorString(e));
     // The launch's shards add up.
     bpsf_work w{};
     unsigned stv = 0;
@@ -1023,26 +1038,26 @@ extern "C" bpsf_status bpsf_decode_plain(bpsf_ctx *c, int64_t n, const uint32_t 
     long long iters_total = 0, trial_runs = 0, failed = 0, cap = 0, cancelled = 0;
     for (int64_t i = 0; i < n; ++i) {
         JobDev job{synd + i * ss, corr + i * cs, conv + i, iters + i, stage ? stage + i : nullptr, 1, ss, cs};
-        cudaError_t e = cudaMemsetAsync(c->d_ctr, 0, sizeof(StreamCounters), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->rec.qseq, 0, 8, s);
+        cudaError_t e = clear_workspace(c, 1, s);
         if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
         BpsfRange shot_range("plain shot");
         StreamDev sdA = bpsf_make_stream(c, job, nullptr, kNoTickets);
+        sdA.ctr = c->w_ctr;
         bpsf_launch_plan(plA, false, &sdA, 1, 1, stream);
-        e = cudaMemcpyAsync(c->h_flag, conv + i, 1, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(c->h_ctr, c->d_ctr, sizeof(StreamCounters), cudaMemcpyDeviceToHost, s);
+        e = cudaMemcpyAsync(c->h_ctr, c->w_ctr, sizeof(StreamCounters), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "plain initial run: %s", cudaGetErrorString(e));
         iters_total += (long long)c->h_ctr->iters_total;
         cap += (long long)c->h_ctr->slot_capacity;
-        if (c->h_flag[0] == 0 && c->p.w > 0) {
+        if (c->h_ctr->rec_count > 0 && c->p.w > 0) {  // the run failed: it has a record
             ++failed;
-            e = cudaMemcpyAsync(c->d_ctr, c->h_preset, sizeof(StreamCounters), cudaMemcpyHostToDevice, s);
+            e = cudaMemcpyAsync(c->w_ctr, c->h_preset, sizeof(StreamCounters), cudaMemcpyHostToDevice, s);
             if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "cudaMemcpyAsync: %s", cudaGetErrorString(e));
             BpsfRange trial_range("plain trial sweep");
             StreamDev sdB = bpsf_make_stream(c, job, nullptr, 0);
+            sdB.ctr = c->w_ctr;
             bpsf_launch_plan(plB, false, &sdB, 1, gridB, stream);
-            e = cudaMemcpyAsync(c->h_ctr, c->d_ctr, sizeof(StreamCounters), cudaMemcpyDeviceToHost, s);
+            e = cudaMemcpyAsync(c->h_ctr, c->w_ctr, sizeof(StreamCounters), cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
             if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "plain trial sweep: %s", cudaGetErrorString(e));
             if (c->h_ctr->status)
@@ -1054,7 +1069,8 @@ extern "C" bpsf_status bpsf_decode_plain(bpsf_ctx *c, int64_t n, const uint32_t 
         }
     }
     c->last = bpsf_work{n, failed, trial_runs, iters_total, iters_total * c->nnz, cap, cancelled};
-    c->d_ctr_last = c->d_ctr;
+    c->d_ctr_last = c->w_ctr;
+    c->last_stream = stream;
     c->last_shards = 1;
     return BPSF_OK;
 }
@@ -1227,16 +1243,15 @@ extern "C" bpsf_status bpsf_decode_multi(int32_t n_jobs, const bpsf_job *jobs, v
         long long cap_s = 0;
         st = bpsf_ensure_workspace_sharded(c, std::max<int64_t>(j.n_shots, 1), shards[k], &cap_s);
         if (st != BPSF_OK) return st;
-        cudaError_t e = cudaMemsetAsync(c->d_ctr, 0, shards[k] * sizeof(StreamCounters), s);
+        cudaError_t e = clear_workspace(c, c->rec.cap, s);
         if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-        st = clear_queue(c, s);
-        if (st != BPSF_OK) return st;
         JobDev job{j.d_synd, j.d_corr, j.d_converged, j.d_iters, j.d_stage, j.n_shots, j.synd_stride_words,
                    j.corr_stride_words};
         bpsf_shard_streams(c, job, shards[k], cap_s, nullptr, sds.data() + at);
         at += shards[k];
         c->last_launch_n = j.n_shots;
-        c->d_ctr_last = c->d_ctr;
+        c->d_ctr_last = c->w_ctr;
+        c->last_stream = stream;
         c->last_shards = shards[k];
     }
     bpsf_launch_plan(pl, false, sds.data(), n_streams, pl.grid, stream);
@@ -1418,6 +1433,7 @@ extern "C" bpsf_status bpsf_selftest_wait(bpsf_ctx *c, int64_t wait_us, void *st
     e = cudaGetLastError();
     if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "kernel launch: %s", cudaGetErrorString(e));
     c->d_ctr_last = c->d_ctr;
+    c->last_stream = stream;
     c->last_shards = 1;
     return bpsf_sync(c, stream);
 }

@@ -31,11 +31,12 @@ struct bpsf_ctx {
     int default_n_trials = 0;
     bpsf::CodeDev code{};
     bpsf::StreamCounters *d_ctr = nullptr;  // per-launch counters, one block per shard (kMaxStreams)
+    bpsf::StreamCounters *w_ctr = nullptr;  // the workspace's counters (batch and plain launches), before its records
+    void *last_stream = nullptr;                 // stream of the most recent launch
     bpsf::StreamCounters *d_ctr_last = nullptr;  // counters of the most recent launch (read by bpsf_sync)
     bpsf::StreamCounters *h_ctr = nullptr;  // pinned copy read by bpsf_sync
     bpsf::StreamCounters *h_preset = nullptr;
-    uint8_t *h_flag = nullptr;              // pinned flag read by the plain form
-    void *d_rec = nullptr;                  // failed-shot records
+    void *d_rec = nullptr;                  // workspace: launch counters, failed-shot records
     bpsf::Records rec{};
     long long rec_cap = 0;
     void *d_host_stage = nullptr;           // device buffers of bpsf_decode_host

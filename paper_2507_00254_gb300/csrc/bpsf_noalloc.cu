@@ -102,8 +102,8 @@ extern "C" bpsf_status bpsf_decode_noalloc(bpsf_ctx *c, int64_t n, const uint32_
     // at zero and every record free.  Every other record field is written
     // before it is read.
     cudaStream_t s = (cudaStream_t)stream;
-    e = cudaMemsetAsync(ctr, 0, sizeof(StreamCounters), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(rec.qseq, 0, 8 * (size_t)ring, s);
+    // (the record numbers are the first array after the counters).
+    e = cudaMemsetAsync(ctr, 0, align256(sizeof(StreamCounters)) + 8 * (size_t)ring, s);
     if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
     JobDev job{synd, corr, conv, iters, stage, n, ss, cs};
     StreamDev sd = bpsf_make_stream(c, job, nullptr, 0);
@@ -119,6 +119,7 @@ extern "C" bpsf_status bpsf_decode_noalloc(bpsf_ctx *c, int64_t n, const uint32_
     e = cudaMemcpyAsync(c->d_ctr, ctr, sizeof(StreamCounters), cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return bpsf_fail(BPSF_ECUDA, "counter copy: %s", cudaGetErrorString(e));
     c->d_ctr_last = c->d_ctr;
+    c->last_stream = stream;
     c->last_shards = 1;
     c->last_launch_n = n;
     return BPSF_OK;
