@@ -1083,11 +1083,12 @@ __device__ __forceinline__ void shot_complete(const StreamDev &sd, long long row
 // One trial of a failed shot is over (run, or cancelled because it cannot
 // win): count it; the last one settles the winner (the minimum key of the
 // shot's converged trials) and completes the shot.
-__device__ __forceinline__ void trial_done(const StreamDev &sd, long long rs, long long row, long long shot) {
+__device__ __forceinline__ void trial_done(const StreamDev &sd, long long rs, long long row, long long shot,
+                                           bool merged) {
     const CodeDev &cd = sd.code;
     const JobDev &job = sd.job;
     const int C = cd.n_trials, Wn = cd.Wn;
-    __threadfence();
+    if (merged) __threadfence();  // its words before its count
     const unsigned d = (atomicAdd(&sd.rec.done[rs], 1u) + 1u) & ((1u << kDoneBits) - 1u);
     if (d == (unsigned)C) {
         __threadfence();
@@ -1151,10 +1152,14 @@ __device__ __forceinline__ void finalize_simple(const StreamDev &sd, TeamMem T, 
         // of the trial's mask.
         uint32_t *ew = T.ebits + s * Wn;
         const unsigned long long mask = __ldg(cd.trial_mask + kidx);
-        for (int j = 0; j < cd.w; ++j) {
-            if (!((mask >> j) & 1ull)) continue;
-            const int b = __ldcg(sd.rec.phi + rs * cd.w + j);
-            ew[b >> 5] ^= 1u << (b & 31);
+        for (int j0 = 0; j0 < cd.w; j0 += 8) {
+            int b[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                b[j] = j0 + j < cd.w && ((mask >> (j0 + j)) & 1ull) ? __ldcg(sd.rec.phi + rs * cd.w + j0 + j) : -1;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (b[j] >= 0) ew[b[j] >> 5] ^= 1u << (b[j] & 31);
         }
         unsigned wsum = 0;
         for (int w = 0; w < Wn; ++w) wsum += __popc(ew[w]);
@@ -1178,7 +1183,7 @@ __device__ __forceinline__ void finalize_simple(const StreamDev &sd, TeamMem T, 
         mg.trials_cancelled += 1;  // stopped: it could not win
     else
         mg.trials_local += 1;
-    trial_done(sd, rs, row, shot);
+    trial_done(sd, rs, row, shot, conv);
 }
 
 // Shots that may be claimed now.
@@ -1199,13 +1204,14 @@ __device__ __forceinline__ long long shots_available(const StreamDev &sd) {
 // p = 0.05 took 2.4 ms, and 1.85 ms with this.
 //
 // When few records are left a block takes no more trials than its idle slots;
-// when less than a launch full of shots is left, no more of them than its idle
-// slots and than about two shares of what is left.  The end of a batch (or all
+// when less than two launches full of shots are left, no more of them than its
+// idle slots and than about two shares of what is left.  The end of a batch (or all
 // of a small one) so spreads over the blocks: 300 [[144]] shots at p = 0.05
 // took 0.37 ms with claims of up to 32 and take 0.34 ms.
 template <bool DEBUG>
 __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qbase, int Q, int qstride, int lane,
-                                         MgrState &mg, int n_empty, int nslots, unsigned long long wait_ns) {
+                                         MgrState &mg, int n_empty, int nslots, unsigned long long head,
+                                         unsigned long long rc, long long shot_next, unsigned long long wait_ns) {
     const CodeDev &cd = sd.code;
     const int Ws = cd.Ws;
     bool got_any = false;
@@ -1213,7 +1219,6 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
     unsigned long long stall = 0ull;
     if (space > 0 && cd.w > 0 && !(sd.flags & kNoTickets)) {
         const int T = cd.n_trials;
-        const unsigned long long head = ld_vol_u64(&sd.ctr->rec_head), rc = ld_vol_u64(&sd.ctr->rec_count);
         int lim = space < 32 ? space : 32;
         if (rc < head + 3ull && lim > n_empty) lim = n_empty;
         if (head < rc && lim > 0) {
@@ -1295,7 +1300,7 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
                         for (int w = 0; w < Ws; ++w) sd.dbg.trial_synd[(shot * T + kidx) * Ws + w] = sy[w];
                 } else {
                     // Early cancel: counted as done, not run.
-                    trial_done(sd, rs, row_of(sd, shot), shot);
+                    trial_done(sd, rs, row_of(sd, shot), shot, false);
                     ++mg.trials_cancelled;
                     e->kind = 0;
                 }
@@ -1321,16 +1326,16 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
         }
     }
     mg.stall_q = stall;
-    if (space > 0) {
+    if (space > 0 && ((sd.flags & kServe) || shot_next < sd.job.n_shots)) {
         long long c0 = 0;
         int got = 0;
         if (lane == 0) {
             const long long avail = shots_available(sd);
-            long long cur = (long long)ld_vol_u64(&sd.ctr->shot_next);
+            long long cur = shot_next;
             for (int att = 0; att < 4 && cur < avail; ++att) {
                 const long long left = avail - cur, grid = (long long)gridDim.x;
                 long long want = space < 32 ? space : 32;
-                if (left < grid * nslots) {
+                if (left < 2 * grid * nslots) {
                     const long long share = 1 + 2 * left / grid;
                     want = want < share ? want : share;
                     want = want < n_empty ? want : n_empty;
@@ -1386,7 +1391,8 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
                              int lane, unsigned long long wait_ns) {
     const CodeDev &cd = sd.code;
     const int qstride = qentry_bytes(cd.Ws);
-    const int nslots = teams * S;
+    const int nslots = teams * S, lgS = __ffs(S) - 1;
+    const bool serve = (sd.flags & kServe) != 0;
     MgrState mg{0, 0, 0u, 0u, 0u, 0ull, 0ull};
     unsigned idle_ns = 32;     // back-off after passes that found nothing to do
     unsigned idle_passes = 0;  // consecutive passes without progress
@@ -1399,7 +1405,7 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
         for (int g0 = 0; g0 < nslots; g0 += 32) {
             const int g = g0 + lane;
             const bool inr = g < nslots;
-            const int t = inr ? g / S : 0, s = inr ? g - t * S : 0;
+            const int t = inr ? g >> lgS : 0, s = g & (S - 1);
             TeamMem T = team_mem(team_base + t * team_bytes, to);
             const int stv = inr ? *vstate(&T.st[s]) : kSlotEmpty;
             const bool fin = inr && *vflag(&T.ob[s].full) != 0;
@@ -1422,6 +1428,9 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
             if (__any_sync(FULLMASK, fin)) progress = true;
         }
         __syncwarp();
+        // The counters that (C) needs, on their way while (B) runs.
+        const unsigned long long rec_head = ld_vol_u64(&sd.ctr->rec_head), rec_count = ld_vol_u64(&sd.ctr->rec_count);
+        const long long shot_next = (long long)ld_vol_u64(&sd.ctr->shot_next);
         // (B) fill empty inboxes from the ready queue: idle slots first (they
         // start at once), then running ones (their next run).  Count the
         // slots left idle with nothing in their inbox.
@@ -1429,7 +1438,7 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
             for (int g0 = 0; g0 < nslots && (pass == 1 || mg.tail > mg.head); g0 += 32) {
                 const int g = g0 + lane;
                 const bool inr = g < nslots;
-                const int t = inr ? g / S : 0, s = inr ? g - t * S : 0;
+                const int t = inr ? g >> lgS : 0, s = g & (S - 1);
                 TeamMem T = team_mem(team_base + t * team_bytes, to);
                 const bool idle = inr && *vstate(&T.st[s]) == kSlotEmpty;
                 const bool open = inr && *vflag(&T.ibf[s]) == 0 && (pass == 1 || idle);
@@ -1452,19 +1461,15 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
         }
         __syncwarp();
         // (C) claim work ahead.
-        if (prefetch<DEBUG>(sd, qbase, Q, qstride, lane, mg, n_empty, nslots, wait_ns)) progress = true;
+        if (prefetch<DEBUG>(sd, qbase, Q, qstride, lane, mg, n_empty, nslots, rec_head, rec_count, shot_next, wait_ns))
+            progress = true;
         // Count finished initial runs once no new shot can be claimed.
-        if (!(sd.flags & kServe)) {
-            int exhausted = 0;
-            if (lane == 0) exhausted = (long long)ld_vol_u64(&sd.ctr->shot_next) >= sd.job.n_shots;
-            exhausted = __shfl_sync(FULLMASK, exhausted, 0);
-            if (exhausted) {
-                const unsigned tot = __reduce_add_sync(FULLMASK, mg.init_local);
-                mg.init_local = 0;
-                if (lane == 0 && tot) {
-                    __threadfence();
-                    atomicAdd(&sd.ctr->init_done, (unsigned long long)tot);
-                }
+        if (!serve && shot_next >= sd.job.n_shots) {
+            const unsigned tot = __reduce_add_sync(FULLMASK, mg.init_local);
+            mg.init_local = 0;
+            if (lane == 0 && tot) {
+                __threadfence();
+                atomicAdd(&sd.ctr->init_done, (unsigned long long)tot);
             }
         }
         // (D) leave when nothing is running, queued, boxed or claimable.
@@ -1472,7 +1477,7 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
             bool any_slot = false;
             for (int g0 = 0; g0 < nslots; g0 += 32) {
                 const int g = g0 + lane;
-                const int t = g < nslots ? g / S : 0, s = g < nslots ? g - t * S : 0;
+                const int t = g < nslots ? g >> lgS : 0, s = g & (S - 1);
                 TeamMem T = team_mem(team_base + t * team_bytes, to);
                 // Read order matters: inbox flag, state, outbox flag (the
                 // team writes state before clearing the inbox flag, and the
