@@ -1203,11 +1203,14 @@ __device__ __forceinline__ long long shots_available(const StreamDev &sd) {
 // the blocks that raced for a failed shot's trials: 30 000 [[144]] shots at
 // p = 0.05 took 2.4 ms, and 1.85 ms with this.
 //
-// When few records are left a block takes no more trials than its idle slots;
-// when less than two launches full of shots are left, no more of them than its
-// idle slots and than about two shares of what is left.  The end of a batch (or all
-// of a small one) so spreads over the blocks: 300 [[144]] shots at p = 0.05
-// took 0.37 ms with claims of up to 32 and take 0.34 ms.
+// While there are fewer trials than the launch has slots (128 when serving,
+// where they go before new shots), a block takes no more of them than its idle
+// slots, and while less than two launches full of shots are left, no more of
+// these than its idle slots and about two shares of what is left.  The end of a
+// batch, or all of a small one, so spreads over the blocks: 300 [[144]] shots
+// at p = 0.05 took 0.37 ms with claims of up to 32 shots and take 0.34 ms;
+// four failed [[254]] shots took 525 us with claims of up to 32 trials (two
+// blocks then ran all 52) and take 102 us.
 template <bool DEBUG>
 __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qbase, int Q, int qstride, int lane,
                                          MgrState &mg, int n_empty, int nslots, unsigned long long head,
@@ -1220,7 +1223,8 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
     if (space > 0 && cd.w > 0 && !(sd.flags & kNoTickets)) {
         const int T = cd.n_trials;
         int lim = space < 32 ? space : 32;
-        if (rc < head + 3ull && lim > n_empty) lim = n_empty;
+        const unsigned long long few = (sd.flags & kServe) ? 128ull : (unsigned long long)gridDim.x * (unsigned)nslots;
+        if (rc < head + 1ull + few / (unsigned)T && lim > n_empty) lim = n_empty;
         if (head < rc && lim > 0) {
             const unsigned long long q = head + (unsigned long long)lane;
             long long rs = (long long)(q & (unsigned long long)(sd.rec.cap - 1));
