@@ -173,6 +173,34 @@ static cudaError_t blocks_per_sm(const void *fn, int block, int smem, int *occ) 
 // given number of blocks per SM is taken at its word.
 constexpr long long kColumnShots = 1500000;
 
+// Long codes (more than kMaxShardNnz edges; up to eight ones per row and three
+// per column): all warps of a block in one team that works on four slots, for
+// any batch.  In teams of four warps with a slot each, three warps waited while
+// one packed and installed 2592 columns.  10^5 shots of the 12-round
+// phenomenological [[144]] at p = q = 0.004: 7.6 ms in such teams, 4.6 with 27
+// warps on four slots, 4.7 with 19 warps, 5.7 with 27 on two slots.
+static bool plan_long(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, bpsf_plan *out, int *variant, int *B,
+                      int *smem, int Q) {
+    int bytes = 0;
+    for (int k = 0; k < n_codes; ++k) {
+        const bpsf_ctx *c = codes[k];
+        if (c->nnz <= kMaxShardNnz || c->dc_max > 8 || c->dv_max > 3 || c->vstride != 4) return false;
+        if (c->code.layered || c->team_only || tunes[k].blocks_per_sm > 0) return false;
+        bytes = std::max(bytes, block_smem_bytes(c->M, c->N, c->code.lay[layout_index(kLongSlots)].P, c->Ws, 4, kLongSlots,
+                                                 1, Q, 0, 2, kPathLong));
+    }
+    if (bytes > codes[0]->smem_optin) return false;
+    for (int k = 0; k < n_codes; ++k) {
+        out->W_code[k] = kMaxLongWarps;
+        out->S_code[k] = kLongSlots;
+        out->teams_code[k] = 1;
+    }
+    *variant = kLongVariant;
+    *B = kMaxLongWarps;
+    *smem = bytes;
+    return true;
+}
+
 static void plan_columns(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, const long long *shots,
                          int dc, int dv, bpsf_plan *out, int *variant, int *B, int *smem, long long *grid_max, int Q) {
     if (kernel_variant_columns(dc, dv, 2) < 0) return;
@@ -198,7 +226,7 @@ static void plan_columns(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning 
         blocks += (runs + teams * S - 1) / (teams * S);
         warps = std::max(warps, W * teams);
         bytes = std::max(bytes, block_smem_bytes(c->M, c->N, c->code.lay[layout_index(S)].P, c->Ws, vstride, S, teams, Q,
-                                                 0, fb, true));
+                                                 0, fb, kPathColumns));
     }
     *variant = kernel_variant_columns(dc, dv, fb);
     *B = warps;
@@ -283,7 +311,8 @@ bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tunin
         if (any_exact) variant = kernel_variant_mixed(variant);
     }
     long long grid_max = 1ll << 30;
-    if (shots && all_regular && !layered)
+    if (shots && plan_long(codes, n_codes, tunes, out, &variant, &B, &smem, Q)) {
+    } else if (shots && all_regular && !layered)
         plan_columns(codes, n_codes, tunes, shots, dc, dv, out, &variant, &B, &smem, &grid_max, Q);
     bpsf_status st = bpsf_ensure_kernel_attrs(variant, c0->smem_optin);
     if (st != BPSF_OK) return st;
@@ -558,16 +587,6 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     for (int e = 0; e < nnz; ++e) csr_col[e] = (uint16_t)c->csr_col[e];
     // Channel LLR (Section II-B, step 1) in double, rounded once to float.
     for (int i = 0; i < N; ++i) lch[i] = (float)std::log((1.0 - priors[i]) / priors[i]);
-    // First iteration's C2V magnitudes: every V2C message is a channel LLR then.
-    std::vector<float> c2v0((size_t)N * vstride, 0.f);
-    const float alpha1 = p.alpha > 0.f ? p.alpha : 0.5f;
-    for (int i = 0; i < N; ++i)
-        for (int k = 0; k < (int)cols[i].size(); ++k) {
-            float m = HUGE_VALF;
-            for (int v : rows[cols[i][k].first])
-                if (v != i) m = std::min(m, lch[v]);
-            c2v0[(size_t)i * vstride + k] = std::min(alpha1 * m, 0x1p100f);
-        }
     cudaGetDevice(&c->device);
     cudaDeviceProp prop;
     cudaError_t e = cudaGetDeviceProperties(&prop, c->device);
@@ -584,7 +603,8 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     for (int i = 0; i < N; ++i)
         for (int k = 0; k < (int)cols[i].size(); ++k) edge_k[row_off[cols[i][k].first] + cols[i][k].second] = k;
     std::vector<std::vector<uint16_t>> lay_vpos(kNumLayouts), lay_var(kNumLayouts);
-    std::vector<std::vector<float>> lay_lch(kNumLayouts);
+    std::vector<std::vector<float>> lay_lch(kNumLayouts), lay_c2v0(kNumLayouts);
+    const float alpha1 = p.alpha > 0.f ? p.alpha : 0.5f;  // damping of a run's first iteration
     int lay_Mp[kNumLayouts];
     for (int li = 0; li < kNumLayouts; ++li) {
         const int S = 1 << li;
@@ -602,6 +622,7 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
         lay_vpos[li].assign((size_t)N * vstride, 0xffff);
         lay_lch[li].assign(PS, 0.f);
         lay_var[li].assign(PS, 0xffff);
+        lay_c2v0[li].assign(PS, 0.f);
         for (int i = 0; i < N; ++i)
             for (int k = 0; k < (int)cols[i].size(); ++k) {
                 const int j = cols[i][k].first, r = rank[row_off[j] + cols[i][k].second];
@@ -612,6 +633,11 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
                 const size_t pos = (size_t)rank[row_off[j] + t] * Mp + j;
                 lay_lch[li][pos] = lch[rows[j][t]];
                 lay_var[li][pos] = (uint16_t)rows[j][t];
+                // Every V2C message of the first iteration is a channel LLR.
+                float m = HUGE_VALF;
+                for (int q = 0; q < (int)rows[j].size(); ++q)
+                    if (q != t) m = std::min(m, lch[rows[j][q]]);
+                lay_c2v0[li][pos] = std::min(alpha1 * m, 0x1p100f);
             }
     }
     // A default set beyond kMaxTrials is left empty: decoding then needs a list.
@@ -649,12 +675,12 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     }
 
     // One allocation for all code arrays.
-    const void *srcs[9] = {row_deg.data(), vchk.data(),      lch.data(),        row_ptr.data(), csr_col.data(),
-                           masks.data(),   layer_ptr.data(), layer_rows.data(), c2v0.data()};
-    const size_t sizes[9] = {(size_t)M, 2 * vchk.size(), 4 * (size_t)N, 2 * (size_t)(M + 1), 2 * (size_t)nnz,
-                             8 * masks.size(), 2 * layer_ptr.size(), 2 * layer_rows.size(), 4 * c2v0.size()};
-    size_t off[9], sz = 0;
-    for (int k = 0; k < 9; ++k) {
+    const void *srcs[8] = {row_deg.data(), vchk.data(), lch.data(), row_ptr.data(), csr_col.data(),
+                           masks.data(), layer_ptr.data(), layer_rows.data()};
+    const size_t sizes[8] = {(size_t)M, 2 * vchk.size(), 4 * (size_t)N, 2 * (size_t)(M + 1), 2 * (size_t)nnz,
+                             8 * masks.size(), 2 * layer_ptr.size(), 2 * layer_rows.size()};
+    size_t off[8], sz = 0;
+    for (int k = 0; k < 8; ++k) {
         off[k] = sz;
         sz += align16(sizes[k]);
     }
@@ -664,7 +690,7 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
         return bpsf_fail(BPSF_ENOMEM, "cudaMalloc(code): %s", cudaGetErrorString(e));
     }
     std::vector<unsigned char> hbuf(sz, 0);
-    for (int k = 0; k < 9; ++k) std::memcpy(hbuf.data() + off[k], srcs[k], sizes[k]);
+    for (int k = 0; k < 8; ++k) std::memcpy(hbuf.data() + off[k], srcs[k], sizes[k]);
     e = cudaMemcpy(c->d_code, hbuf.data(), sz, cudaMemcpyHostToDevice);
     unsigned char *base = (unsigned char *)c->d_code;
     CodeDev &cd = c->code;
@@ -695,16 +721,16 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     cd.n_layers = n_layers;
     cd.layer_ptr = (const uint16_t *)(base + off[6]);
     cd.layer_rows = (const uint16_t *)(base + off[7]);
-    cd.c2v0 = (const float *)(base + off[8]);
     c->default_n_trials = c->n_trials;
     // The per-slot-count layouts: one allocation.
     {
         size_t lsz = 0;
-        size_t lo[kNumLayouts][3];
+        size_t lo[kNumLayouts][4];
         for (int li = 0; li < kNumLayouts; ++li) {
             lo[li][0] = lsz; lsz += align16(2 * lay_vpos[li].size());
             lo[li][1] = lsz; lsz += align16(4 * lay_lch[li].size());
             lo[li][2] = lsz; lsz += align16(2 * lay_var[li].size());
+            lo[li][3] = lsz; lsz += align16(4 * lay_c2v0[li].size());
         }
         if (e == cudaSuccess) e = cudaMalloc(&c->d_layouts, lsz);
         if (e == cudaSuccess) {
@@ -713,6 +739,7 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
                 std::memcpy(lb.data() + lo[li][0], lay_vpos[li].data(), 2 * lay_vpos[li].size());
                 std::memcpy(lb.data() + lo[li][1], lay_lch[li].data(), 4 * lay_lch[li].size());
                 std::memcpy(lb.data() + lo[li][2], lay_var[li].data(), 2 * lay_var[li].size());
+                std::memcpy(lb.data() + lo[li][3], lay_c2v0[li].data(), 4 * lay_c2v0[li].size());
             }
             e = cudaMemcpy(c->d_layouts, lb.data(), lsz, cudaMemcpyHostToDevice);
             unsigned char *lbase = (unsigned char *)c->d_layouts;
@@ -723,6 +750,7 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
                 ly.vpos = (const uint16_t *)(lbase + lo[li][0]);
                 ly.lch_pos = (const float *)(lbase + lo[li][1]);
                 ly.pos_var = (const uint16_t *)(lbase + lo[li][2]);
+                ly.c2v0 = (const float *)(lbase + lo[li][3]);
             }
             bpsf_activate_layout(cd, 1);
         }

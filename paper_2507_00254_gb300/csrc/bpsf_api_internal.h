@@ -125,6 +125,7 @@ inline void bpsf_activate_layout(bpsf::CodeDev &cd, int S) {
     cd.vpos = ly.vpos;
     cd.lch_pos = ly.lch_pos;
     cd.pos_var = ly.pos_var;
+    cd.c2v0 = ly.c2v0;
 }
 
 // A context with trials (w > 0) decodes only with a non-empty trial set.

@@ -55,9 +55,15 @@ __device__ __forceinline__ int first_cap(const SlotState *st, unsigned run, int 
 }
 
 // sd, to: the block's copies in shared memory; tb: the team's offset there.
-template <int DC, int DV, int DVS, int V, bool DEBUG, int FB>
-__device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffsets &to, BlockHdr *hdr, const int tb,
-                                            const int W, const int tid, const int bar_id) {
+// LONG: codes with more columns than a team has lanes, of at most DC ones per
+// row and DV per column.  Lanes loop over columns and rows, whose tables and
+// flip words are in shared memory, and the syndrome bits of 32 / V rows share a
+// word (bit j*V + c, as in the team path): fewer words to look at, and few
+// decisions change.
+template <int DC, int DV, int DVS, int V, bool LONG, bool DEBUG, int FB>
+__device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffsets &to, BlockHdr *hdr,
+                                            const LayoutMem &L, const int tb, const int W, const int tid_,
+                                            const int bar_id) {
     typedef typename VecF<V>::T VT;
     typedef FlipPack<FB, V> FP;
     constexpr int lgS = V == 4 ? 2 : V - 1;
@@ -67,27 +73,30 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
     typedef typename VecF<CV>::T CT;
     const CodeDev &cd = sd.code;
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = tid & 31;
+    const int tid = tid_, nth_ = 32 * W, nth = nth_, lane = tid & 31;
     const bool sw = (tid >> 5) == W - 1;  // service warp
-    const int M = keep(cd.M);
-    const bool col_on = tid < cd.N, row_on = tid < CG * M;
-    const int o_mism = keep(tb + to.mism);
-    // The lane's row and its slots there.
-    const int mrow = tb + to.m + (row_on ? tid : 0) * (int)sizeof(CT);
+    const int M = keep(cd.M), N = keep(cd.N);
+    const int nw = LONG ? keep(((M << lgS) + 31) >> 5) : M;  // residual words
+    const int o_mism = keep(tb + to.mism), o_m = keep(tb + to.m), o_flips = keep(tb + to.flips);
+    const int o_syn = keep(tb + to.syn);
     const int mstride = keep(cd.Mp * (int)sizeof(VT));
+    // !LONG: the lane's row part (seeds) and column: message and residual word
+    // (byte offsets in shared memory), channel LLR, flip words.
     float seed[CV];
 #pragma unroll
     for (int c = 0; c < CV; ++c) seed[c] = 0.f;
-    // The lane's column: messages, residual words (byte offsets in shared memory).
     int mcol[DV], res[DV];
-#pragma unroll
-    for (int d = 0; d < DV; ++d) {
-        const int e = (col_on ? tid : 0) * DVS + d;
-        mcol[d] = tb + to.m + (int)cd.vpos[e] * (int)sizeof(VT);
-        res[d] = o_mism + 4 * (int)cd.vchk[e];
-    }
-    const float lc = cd.lch[col_on ? tid : 0];
+    float lc = 0.f;
     typename FP::U fw = typename FP::U();
+    if (!LONG) {
+        const int i = tid < N ? tid : 0;
+#pragma unroll
+        for (int d = 0; d < DV; ++d) {
+            mcol[d] = o_m + (int)cd.vpos[i * DVS + d] * (int)sizeof(VT);
+            res[d] = o_mism + 4 * (int)cd.vchk[i * DVS + d];
+        }
+        lc = cd.lch[i];
+    }
     typename FP::D on = FP::on(0u);  // the running slots' decision bits
     const bool adaptive = keep(!(cd.alpha > 0.f));
     const bool first_rule = keep(cd.select == 1);
@@ -112,27 +121,54 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
         if (run != 0u) {
             // C phase; the decision on the previous iteration is made beside it.
             uint4 w4 = make_uint4(0u, 0u, 0u, 0u);
-            if (4 * lane < M) w4 = *reinterpret_cast<const uint4 *>(smem + o_mism + 16 * lane);
+            if (!LONG && 4 * lane < nw) w4 = *reinterpret_cast<const uint4 *>(smem + o_mism + 16 * lane);
             if (adaptive) {
 #pragma unroll
                 for (int c = 0; c < CV; ++c) al[c] = __fmaf_rn(al[c], 0.5f, 0.5f);
             }
-            if (row_on) {
-                float x[DC][CV];
+            auto row_part = [&](int task) {
+                const int deg = LONG ? (int)L.row_deg[task / CG] : DC;
+                unsigned char *row = smem + o_m + task * (int)sizeof(CT);
+                float x[DC][CV], sd_[CV];
 #pragma unroll
-                for (int k = 0; k < DC; ++k) vload<CV>(x[k], reinterpret_cast<const CT *>(smem + mrow + k * mstride));
+                for (int k = 0; k < DC; ++k) {
+                    if (!LONG || k < deg) {
+                        vload<CV>(x[k], reinterpret_cast<const CT *>(row + k * mstride));
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < CV; ++c) x[k][c] = __int_as_float(0x7f800000);
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < CV; ++c) sd_[c] = seed[c];
+                if (LONG) {
+                    const int b = task * CV;  // the part's first syndrome bit
+                    row_seed<CV, true>(sd_, *reinterpret_cast<const uint32_t *>(smem + o_syn + (b >> 5) * 4) >> (b & 31));
+                }
 #pragma unroll
                 for (int k = 0; k < DC; ++k) vmul<CV>(x[k], x[k], al);
-                row_outputs<DC, CV>(x, seed);
+                row_outputs<DC, CV>(x, sd_);
 #pragma unroll
-                for (int k = 0; k < DC; ++k) vstore<CV>(reinterpret_cast<CT *>(smem + mrow + k * mstride), x[k]);
+                for (int k = 0; k < DC; ++k)
+                    if (!LONG || k < deg) vstore<CV>(reinterpret_cast<CT *>(row + k * mstride), x[k]);
+            };
+            if (LONG) {
+#pragma unroll 1
+                for (int task = tid; task < CG * M; task += nth) row_part(task);
+                if (4 * lane < nw) w4 = *reinterpret_cast<const uint4 *>(smem + o_mism + 16 * lane);
+            } else if (tid < CG * M) {
+                row_part(tid);
             }
             unsigned acc = (w4.x | w4.y) | (w4.z | w4.w);
-            for (int j = 4 * lane + 128; j < M; j += 128) {
+            for (int j = 4 * lane + 128; j < nw; j += 128) {
                 w4 = *reinterpret_cast<const uint4 *>(smem + o_mism + 4 * j);
                 acc |= (w4.x | w4.y) | (w4.z | w4.w);
             }
-            const unsigned nconv = __reduce_or_sync(FULLMASK, acc);
+            if (LONG) {
+#pragma unroll
+                for (int sh = 16; sh >= V; sh >>= 1) acc |= acc >> sh;
+            }
+            const unsigned nconv = __reduce_or_sync(FULLMASK, acc) & full;
             if ((run & ~nconv) || tt >= next_cap) {
                 SlotState *st = reinterpret_cast<SlotState *>(smem + tb + to.state);
                 const bool mine = (run >> lane) & 1u;
@@ -148,7 +184,9 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
             }
         }
         if (run == 0u || (rest & full) || ((tt & 3) == 0 && (run != full || first_rule))) {
-            // Service step.
+            // Service step.  (Its index arithmetic is kept from moving out of the loop,
+            // where it would hold registers all the time.)
+            const int tid = keep(tid_), nth = keep(nth_), lane = tid & 31;
             const TeamMem T = team_mem(smem + tb, to);
             unsigned pend = rest & full, pconv = (rest >> 8) & full, initm = rest >> 16;
             if (sw) {
@@ -211,17 +249,28 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
             const unsigned pk = pend & (ev >> 16);
             const unsigned inst = (full & ~run & ~(pend & ~pk)) & (ev >> 8);
             if (pk) {
-                // Pack: a warp's columns are one word of a finished slot's decision.
-#pragma unroll
-                for (int c = 0; c < V; ++c) {
-                    if (!((pk >> c) & 1u)) continue;
+                // Pack: a warp's k-th columns are one word of a finished slot's decision.
+#pragma unroll 1
+                for (unsigned m = pk; m; m &= m - 1u) {
+                    const int c = __ffs(m) - 1;
                     const bool counts = ((initm & ~pconv) >> c) & 1u;
-                    const unsigned f = flip_field<FB, V>(fw, c);
-                    const unsigned word = __ballot_sync(FULLMASK, col_on && flip_dec<FB>(f) != 0u);
-                    if (lane == 0 && col_on) T.ebits[c * cd.Wn + (tid >> 5)] = word;
-                    if (col_on && counts) flipw<FB>(T)[(tid << lgS) + c] = (typename FlipW<FB>::W)f;
-                    if (DEBUG && sd.dbg.flips && col_on && ((initm >> c) & 1u))
-                        sd.dbg.flips[T.st[c].shot * cd.N + tid] = (uint16_t)flip_count<FB>(f);
+                    // A converged initial run's decision is the shot's result.
+                    uint32_t *words = T.ebits + c * cd.Wn;
+                    if ((initm & pconv) >> c & 1u) words = sd.job.corr + row_of(sd, T.st[c].shot) * sd.job.corr_stride;
+#pragma unroll 2
+                    for (int i0 = tid - lane; i0 < N; i0 += nth) {
+                        const int i = i0 + lane;
+                        unsigned f = 0u;
+                        if (!LONG)
+                            f = flip_field<FB, V>(fw, c);
+                        else if (i < N)
+                            f = (unsigned)flipw<FB>(T)[(i << lgS) + c];
+                        const unsigned word = __ballot_sync(FULLMASK, i < N && flip_dec<FB>(f) != 0u);
+                        if (lane == 0) words[i >> 5] = word;
+                        if (!LONG && i < N && counts) flipw<FB>(T)[(i << lgS) + c] = (typename FlipW<FB>::W)f;
+                        if (DEBUG && sd.dbg.flips && i < N && ((initm >> c) & 1u))
+                            sd.dbg.flips[T.st[c].shot * N + i] = (uint16_t)flip_count<FB>(f);
+                    }
                 }
                 team_sync(W, bar_id);
                 if (sw) {
@@ -237,7 +286,7 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                         const int c = __ffs(m) - 1;
                         const SlotState *ss = &T.st[c];
                         if (((initm >> c) & 1u) && ss->outcome == 2 && cd.w > 0)
-                            publish_failure<DEBUG, FB, true>(sd, T, lgS, c, lane, hdr->wait_ns);
+                            publish_failure<DEBUG, FB, !LONG>(sd, T, lgS, c, lane, hdr->wait_ns);
                         if (lane == 0) {
                             OutBox *ob = &T.ob[c];
                             ob->kind = ss->kind;
@@ -256,39 +305,69 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                         __syncwarp();
                     }
                 }
+                // A failed run's record is made from the syndrome and flip words that an
+                // install rewrites (!LONG: its words are the service warp's own).
+                if (LONG && (pk & initm & ~pconv)) team_sync(W, bar_id);
                 pend &= ~pk;
             }
             if (inst) {
                 __threadfence_block();  // the inbox items are visible
                 unsigned live = 0u;
-                unsigned mis = tid < M ? T.mism[tid] : 0u;
-#pragma unroll
-                for (int c = 0; c < V; ++c) {
-                    if (!((inst >> c) & 1u)) continue;
+                unsigned mis = !LONG && tid < M ? T.mism[tid] : 0u;
+#pragma unroll 1
+                for (unsigned m = inst; m; m &= m - 1u) {
+                    const int c = __ffs(m) - 1;
                     const QEntry *e = reinterpret_cast<const QEntry *>(T.ib + c * T.ibstride);
                     const uint32_t *src = reinterpret_cast<const uint32_t *>(T.ib + c * T.ibstride + sizeof(QEntry));
                     const int kind = e->kind;
                     if (kind == 0) continue;
                     live |= 1u << c;
                     initm = kind == 1 ? initm | (1u << c) : initm & ~(1u << c);
-                    if (tid < M) mis = (mis & ~(1u << c)) | (((src[tid >> 5] >> (tid & 31)) & 1u) << c);
-                    if (row_on && c / CV == tid % CG) {
-                        // The stored C2V messages carry the opposite sign.
-                        const int j = tid / CG;
-                        seed[c % CV] = __uint_as_float((((src[j >> 5] >> (j & 31)) & 1u) ? 0u : 0x80000000u) | 0x71800000u);
-                        if (adaptive) al[c % CV] = 0.5f;
-                    }
-                    flip_clear<FB, V>(fw, c);
-                    if (col_on) {
+                    if (!LONG) {
+                        if (tid < M) mis = (mis & ~(1u << c)) | (((src[tid >> 5] >> (tid & 31)) & 1u) << c);
+                        if (tid < CG * M && c / CV == tid % CG) {
+                            // The stored C2V messages carry the opposite sign.
+                            const int j = tid / CG;
+                            const unsigned b = (src[j >> 5] >> (j & 31)) & 1u;
 #pragma unroll
-                        for (int d = 0; d < DV; ++d) {
-                            const int j = (res[d] - o_mism) >> 2;
-                            const float r = __ldg(cd.c2v0 + tid * DVS + d);
-                            reinterpret_cast<float *>(smem + mcol[d])[c] = ((src[j >> 5] >> (j & 31)) & 1u) ? r : -r;
+                            for (int h = 0; h < CV; ++h)
+                                if (c % CV == h) seed[h] = __uint_as_float((b ? 0u : 0x80000000u) | 0x71800000u);
                         }
+                        flip_clear<FB, V>(fw, c);
+                    } else {
+                        // Word w: rows w * 32/V .., slot c at bits c, c + V, ...
+                        constexpr int per = 32 / V;
+                        for (int w = tid; w < nw; w += nth) {
+                            const unsigned b = src[(w * per) >> 5] >> ((w * per) & 31);
+                            unsigned keep_ = 0u, put = 0u;
+#pragma unroll
+                            for (int j = 0; j < per; ++j) {
+                                keep_ |= 1u << (j * V);
+                                put |= (w * per + j < M ? (b >> j) & 1u : 0u) << (j * V);
+                            }
+                            T.mism[w] = (T.mism[w] & ~(keep_ << c)) | (put << c);
+                            T.syn[w] = (T.syn[w] & ~(keep_ << c)) | (put << c);
+                        }
+                        for (int i = tid; i < N; i += nth) flipw<FB>(T)[(i << lgS) + c] = 0;
+                    }
+                    if (c / CV == tid % CG) {
+#pragma unroll
+                        for (int h = 0; h < CV; ++h)
+                            if (adaptive && c % CV == h) al[h] = 0.5f;
+                    }
+                    // The row's first C2V messages, by its syndrome bit.
+                    for (int j = tid; j < M; j += nth) {
+                        const unsigned flip = ((src[j >> 5] >> (j & 31)) & 1u) ? 0u : 0x80000000u;
+                        const int dj = LONG ? (int)L.row_deg[j] : DC;
+                        float *msg = reinterpret_cast<float *>(smem + o_m) + j * V + c;
+#pragma unroll
+                        for (int k = 0; k < DC; ++k)
+                            if (!LONG || k < dj)
+                                msg[k * (mstride >> 2)] =
+                                    __uint_as_float(__float_as_uint(__ldg(cd.c2v0 + k * cd.Mp + j)) ^ flip);
                     }
                     if (sw) {
-                        for (int w = lane; w < cd.Ws; w += 32) T.syn[c * cd.Ws + w] = src[w];
+                        for (int w = lane; !LONG && w < cd.Ws; w += 32) T.syn[c * cd.Ws + w] = src[w];
                         if (lane == 0) {
                             SlotState *ss = &T.st[c];
                             ss->kind = kind;
@@ -301,7 +380,7 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                         }
                     }
                 }
-                if (tid < M) T.mism[tid] = mis;
+                if (!LONG && tid < M) T.mism[tid] = mis;
                 team_sync(W, bar_id);
                 if (sw && lane == 0) {
                     // RUNNING before the inbox reads empty: the manager's exit test
@@ -327,13 +406,20 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
         } else {
             team_sync(W, bar_id);
         }
-        // V phase.
-        if (col_on) {
+        // V phase.  mp: the messages' places, -1 where the column has no such edge.
+        auto column = [&](int i, const int (&mp)[DV], float l, typename FP::U &f) {
             float r[DV][V], pre[V], nl[V];
 #pragma unroll
-            for (int d = 0; d < DV; ++d) vload<V>(r[d], reinterpret_cast<const VT *>(smem + mcol[d]));
+            for (int d = 0; d < DV; ++d) {
+                if (!LONG || mp[d] >= 0) {
+                    vload<V>(r[d], reinterpret_cast<const VT *>(smem + mp[d]));
+                } else {
 #pragma unroll
-            for (int c = 0; c < V; ++c) pre[c] = lc;
+                    for (int c = 0; c < V; ++c) r[d][c] = 0.f;
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < V; ++c) pre[c] = l;
 #pragma unroll
             for (int d = 0; d < DV; ++d) {
                 float acc[V];
@@ -345,20 +431,43 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                     vsub<V>(pre, pre, r[d]);
                 else
                     vsub<V>(nl, r[d], pre);  // -l_out
-                vstore<V>(reinterpret_cast<VT *>(smem + mcol[d]), acc);
+                if (!LONG || mp[d] >= 0) vstore<V>(reinterpret_cast<VT *>(smem + mp[d]), acc);
             }
             if (DEBUG && sd.dbg.lout) {
                 const SlotState *st = reinterpret_cast<const SlotState *>(smem + tb + to.state);
 #pragma unroll
                 for (int c = 0; c < V; ++c)
-                    if (((run & (rest >> 16)) >> c) & 1u) sd.dbg.lout[st[c].shot * cd.N + tid] = __fsub_rn(0.f, nl[c]);
+                    if (((run & (rest >> 16)) >> c) & 1u) sd.dbg.lout[st[c].shot * N + i] = __fsub_rn(0.f, nl[c]);
             }
-            const typename FP::D dd = FP::diff(nl, fw, on);
+            const typename FP::U f0 = f;
+            const typename FP::D dd = FP::diff(nl, f0, on);
             if (FP::any(dd)) {
-                fw = FP::bump(fw, dd);
+                f = FP::bump(f0, dd);
                 const unsigned bm = FP::slots(dd);
 #pragma unroll
-                for (int d = 0; d < DV; ++d) atomicXor(reinterpret_cast<uint32_t *>(smem + res[d]), bm);
+                for (int d = 0; d < DV; ++d) {
+                    if (!LONG) {
+                        atomicXor(reinterpret_cast<uint32_t *>(smem + res[d]), bm);
+                    } else if (mp[d] >= 0) {
+                        const int b = (int)__ldg(cd.vchk + i * DVS + d) << lgS;
+                        atomicXor(reinterpret_cast<uint32_t *>(smem + o_mism) + (b >> 5), bm << (b & 31));
+                    }
+                }
+            }
+        };
+        if (!LONG) {
+            if (tid < N) column(tid, mcol, lc, fw);
+        } else {
+            typename FP::U *fl = reinterpret_cast<typename FP::U *>(smem + o_flips);
+#pragma unroll 1
+            for (int i = tid; i < N; i += nth) {
+                static_assert(!LONG || DVS == 4, "a column's places are one 64-bit word");
+                const uint2 raw = *reinterpret_cast<const uint2 *>(L.vpos + i * DVS);
+                const unsigned p[4] = {raw.x & 0xffffu, raw.x >> 16, raw.y & 0xffffu, raw.y >> 16};
+                int mp[DV];
+#pragma unroll
+                for (int d = 0; d < DV; ++d) mp[d] = p[d & 3] == 0xffffu ? -1 : o_m + (int)p[d & 3] * (int)sizeof(VT);
+                column(i, mp, L.lch[i], fl[i]);
             }
         }
         ++tt;

@@ -13,6 +13,10 @@ constexpr int kMaxStreams = 16;   // codes per launch
 constexpr int kMaxComputeWarps = 15;  // plus one manager warp: <= 512 threads per block
 constexpr int kMaxColumnWarps = 19;   // column path: with the manager 20 warps, 96 registers a thread
 constexpr int kColumnThreads = 32 * (kMaxColumnWarps + 1);
+constexpr int kMaxLongWarps = 27;      // long codes: with the manager 28 warps, 72 registers a thread
+constexpr int kLongThreads = 32 * (kMaxLongWarps + 1);
+constexpr int kLongSlots = 4;          // slots of its teams
+constexpr int kLongVariant = 12;
 constexpr int kMaxNamedTeams = 15;    // named barriers 1..15 for multi-warp teams
 constexpr int kDVP = 4;           // column entries stored per variable for dv <= 4 codes
 
@@ -46,6 +50,7 @@ struct LayoutS {
     const uint16_t *vpos;     // N x vstride positions
     const float *lch_pos;     // P, channel LLR of the variable at each position
     const uint16_t *pos_var;  // P, variable at each position (0xffff: unused)
+    const float *c2v0;        // P, magnitude of the first iteration's C2V message at each position
 };
 constexpr int kNumLayouts = 6;  // S = 1, 2, 4, 8, 16, 32
 
@@ -59,13 +64,13 @@ struct CodeDev {
     const uint16_t *vpos;        // N x vstride, message positions (0xffff padding), active layout
     const uint16_t *vchk;        // N x vstride, check indices
     const float *lch;            // N, channel LLRs (FP32)
-    const float *c2v0;           // N x vstride, magnitude of the first iteration's C2V messages
     const float *lch_pos;        // P, channel LLR of the variable at each position, active layout
     const uint16_t *row_ptr;     // M+1, CSR (syndrome kernel)
     const uint16_t *csr_col;     // nnz
     const unsigned long long *trial_mask;  // n_trials subset masks over Phi (bit j selects Phi[j]), list order
     int Mp;                      // rank stride of the active layout (see LayoutS)
     const uint16_t *pos_var;     // active layout: variable at each position
+    const float *c2v0;           // active layout: magnitude of the first iteration's C2V messages
     LayoutS lay[kNumLayouts];    // per slot count; a launch activates the one of its S
     int layered;                 // 1: layered schedule
     int n_layers;
@@ -187,21 +192,25 @@ __host__ __device__ inline int align_up(int x, int a) { return (x + a - 1) / a *
 
 constexpr int kBlockHeaderBytes = 64;
 
+// How a launch works on its codes: teams of warps that serve a few slots a
+// lane; a lane per column; lanes that loop over the columns of a long code.
+enum : int { kPathTeams = 0, kPathColumns = 1, kPathLong = 2 };
+
 struct LayoutOffsets {
     int row_deg, vpos, lch, lch_pos, total;
 };
 
-__host__ __device__ inline LayoutOffsets layout_offsets(int M, int N, int vstride, int P, bool cols = false) {
+__host__ __device__ inline LayoutOffsets layout_offsets(int M, int N, int vstride, int P, int path = kPathTeams) {
     LayoutOffsets o;
     int p = 0;
-    if (cols) {  // the column path keeps its tables in registers
+    if (path == kPathColumns) {  // tables in registers
         o.row_deg = o.vpos = o.lch = o.lch_pos = o.total = 0;
         return o;
     }
     o.row_deg = p;  p = align_up(p + M, 16);
     o.vpos = p;     p = align_up(p + 2 * N * vstride, 16);
     o.lch = p;      p = align_up(p + 4 * N, 16);
-    o.lch_pos = p;  p = align_up(p + 4 * P, 16);
+    o.lch_pos = p;  p = align_up(p + (path == kPathTeams ? 4 * P : 0), 16);
     o.total = p;
     return o;
 }
@@ -304,15 +313,16 @@ constexpr int kDescriptorBytes = kStreamBytes + 64;
 static_assert(sizeof(TeamOffsets) <= 64, "team offsets fit their copy");
 
 __host__ __device__ inline TeamOffsets team_offsets(int S, int M, int N, int P, int Ws, int layered, int fb = 2,
-                                                    bool cols = false) {
+                                                    int path = kPathTeams) {
     TeamOffsets o;
     const int sw = (S * M + 31) / 32;
     int p = 0;
     o.ctl = p;     p += 64;
     o.state = p;   p += (int)sizeof(SlotState) * S;
     o.outbox = p;  p += (int)sizeof(OutBox) * S;
-    o.syn = p;     p += cols ? align_up(4 * S * Ws, 16) : 4 * sw;
-    o.mism = p;    p += cols ? align_up(4 * M, 16) : 4 * sw;
+    // (column path: syn S x Ws words, one residual word per row)
+    o.syn = p;     p += path == kPathTeams ? 4 * sw : align_up(4 * (path == kPathColumns ? S * Ws : sw), 16);
+    o.mism = p;    p += path == kPathTeams ? 4 * sw : align_up(4 * (path == kPathColumns ? M : sw), 16);
     o.ebits = p;   p += 4 * S * ((N + 31) / 32);
     o.inflag = p;  p = align_up(p + 4 * S, 16);
     o.ibstride = qentry_bytes(Ws);
@@ -325,9 +335,9 @@ __host__ __device__ inline TeamOffsets team_offsets(int S, int M, int N, int P, 
 }
 
 __host__ __device__ inline int block_smem_bytes(int M, int N, int P, int Ws, int vstride, int S, int teams, int Q,
-                                                int layered, int fb = 2, bool cols = false) {
-    return kBlockHeaderBytes + (cols ? kDescriptorBytes : 0) + layout_offsets(M, N, vstride, P, cols).total + Q * qentry_bytes(Ws) +
-           teams * team_offsets(S, M, N, P, Ws, layered, fb, cols).total;
+                                                int layered, int fb = 2, int path = kPathTeams) {
+    return kBlockHeaderBytes + (path != kPathTeams ? kDescriptorBytes : 0) + layout_offsets(M, N, vstride, P, path).total + Q * qentry_bytes(Ws) +
+           teams * team_offsets(S, M, N, P, Ws, layered, fb, path).total;
 }
 
 // Arguments of one persistent launch: the streams (codes) it serves, by value.

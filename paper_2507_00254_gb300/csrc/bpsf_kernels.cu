@@ -25,6 +25,7 @@ KernelFn kernel_fn_v8(bool debug, bool lay);
 KernelFn kernel_fn_v9(bool debug, bool lay);
 KernelFn kernel_fn_v10(bool debug, bool lay);
 KernelFn kernel_fn_v11(bool debug, bool lay);
+KernelFn kernel_fn_v12(bool debug, bool lay);
 
 // ---------------------------------------------------------------------------
 // Variants and launch helpers.
@@ -40,7 +41,8 @@ struct Variant {
 // kernel_variant_full_regs, kernel_variant_byte_flips and
 // kernel_variant_mixed).
 static const Variant kVariants[] = {{6, 4, 3}, {6, 4, 0}, {8, 4, 0}, {16, 8, 0}, {32, 16, 0}, {6, 4, 3}, {6, 4, 3},
-                                    {8, 4, 0}, {6, 4, 3}, {6, 4, 3}, {10, 8, 5}, {10, 8, 5}};
+                                    {8, 4, 0}, {6, 4, 3}, {6, 4, 3}, {10, 8, 5}, {10, 8, 5},
+                                    {8, 4, 0}};
 static const int kNumVariants = 5;
 
 // Smallest variant that fits.  The exact-degree variant serves codes with
@@ -73,7 +75,8 @@ static KernelFn kernel_fn(int variant, bool debug, bool lay) {
         case 8: return kernel_fn_v8(debug, lay);
         case 9: return kernel_fn_v9(debug, lay);
         case 10: return kernel_fn_v10(debug, lay);
-        default: return kernel_fn_v11(debug, lay);
+        case 11: return kernel_fn_v11(debug, lay);
+        default: return kernel_fn_v12(debug, lay);
     }
 }
 

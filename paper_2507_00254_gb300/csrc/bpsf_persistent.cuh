@@ -1034,6 +1034,11 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
     }
 }
 
+// The output row of a shot.
+__device__ __forceinline__ long long row_of(const StreamDev &sd, long long shot) {
+    return (sd.flags & kServe) ? (shot % sd.serve.rows) : shot;
+}
+
 }  // namespace bpsf
 
 #include "bpsf_columns.cuh"
@@ -1067,9 +1072,6 @@ __device__ __forceinline__ uint32_t *qsyn(QEntry *e) {
 __device__ __forceinline__ unsigned slot_word(const uint32_t *ebits, int Wn, int s, int w) { return ebits[s * Wn + w]; }
 
 
-__device__ __forceinline__ long long row_of(const StreamDev &sd, long long shot) {
-    return (sd.flags & kServe) ? (shot % sd.serve.rows) : shot;
-}
 
 // One shot's final output is out: when serving, post it to the row's
 // completion word (the outputs live in host-mapped memory, hence the
@@ -1119,8 +1121,9 @@ __device__ __forceinline__ bool trial_cannot_win(const StreamDev &sd, long long 
 }
 
 // Lane-parallel write-out of outboxes that need no warp cooperation:
-// converged or uncorrectable initial runs, and trial runs.
-template <bool DEBUG>
+// converged or uncorrectable initial runs, and trial runs.  (COLS: a converged
+// initial run's words are out already.)
+template <bool DEBUG, bool COLS>
 __device__ __forceinline__ void finalize_simple(const StreamDev &sd, TeamMem T, int s, MgrState &mg) {
     const CodeDev &cd = sd.code;
     const JobDev &job = sd.job;
@@ -1136,7 +1139,8 @@ __device__ __forceinline__ void finalize_simple(const StreamDev &sd, TeamMem T, 
         // output (written by its team before it published the trials).
         if (!conv && cd.w > 0) return;
         uint32_t *out = job.corr + row * job.corr_stride;
-        for (int w = 0; w < Wn; ++w) out[w] = slot_word(T.ebits, Wn, s, w);
+        if (!COLS || !conv)
+            for (int w = 0; w < Wn; ++w) out[w] = slot_word(T.ebits, Wn, s, w);
         job.conv[row] = conv ? 1 : 0;
         job.iters[row] = (int16_t)(conv ? iter : cd.max_iter);
         if (job.stage) job.stage[row] = conv ? 0 : 2;
@@ -1372,15 +1376,26 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
         __syncwarp();
         if (lane < got) {
             const long long shot = c0 + lane;
-            const long long row = row_of(sd, shot);
             QEntry *e = qentry(qbase, (mg.tail + lane) % Q, qstride);
             e->kind = 1;
             e->kidx = 0;
             e->rec = -1;
             e->shot = shot;
-            const uint32_t *src = sd.job.synd + row * sd.job.synd_stride;
-            uint32_t *sy = qsyn(e);
-            for (int w = 0; w < Ws; ++w) sy[w] = __ldcg(src + w);
+        }
+        // The syndromes' words, spread over the lanes; four loads of a lane are under way at a time.
+        const int words = got * Ws;
+        for (int k0 = lane; k0 < words; k0 += 128) {
+            uint32_t v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = k0 + 32 * u, sh = k / Ws;
+                if (k < words) v[u] = __ldcg(sd.job.synd + row_of(sd, c0 + sh) * sd.job.synd_stride + (k - sh * Ws));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = k0 + 32 * u, sh = k / Ws;
+                if (k < words) qsyn(qentry(qbase, (mg.tail + sh) % Q, qstride))[k - sh * Ws] = v[u];
+            }
         }
         __syncwarp();
         mg.tail += got;
@@ -1389,7 +1404,7 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
     return got_any;
 }
 
-template <bool DEBUG>
+template <bool DEBUG, bool COLS>
 __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned char *team_base, int team_bytes,
                              const TeamOffsets &to, int teams, int S, unsigned char *qbase, int Q, BlockHdr *hdr,
                              int lane, unsigned long long wait_ns) {
@@ -1423,7 +1438,7 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
                 if (T.st[s].cancel != key && trial_cannot_win(sd, T.st[s].rec, kidx))
                     *reinterpret_cast<volatile long long *>(&T.st[s].cancel) = key;
             }
-            if (fin) finalize_simple<DEBUG>(sd, T, s, mg);
+            if (fin) finalize_simple<DEBUG, COLS>(sd, T, s, mg);
             __syncwarp();
             if (fin) {
                 __threadfence_block();
@@ -1557,7 +1572,8 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
 // keep their specialised path in a launch that mixes them with codes of
 // wider rows (the layouts agree: both have column tables of width DVS).
 template <int DC, int DVS, int DVX, bool DEBUG, int MINB, bool LAY, int FB = 2, bool MIX = false, bool COLS = false>
-__global__ void __launch_bounds__(COLS ? kColumnThreads : 512, MINB) bpsf_persistent(const __grid_constant__ KernelParams kp) {
+__global__ void __launch_bounds__(COLS ? (DVX > 0 ? kColumnThreads : kLongThreads) : 512, MINB) bpsf_persistent(const __grid_constant__ KernelParams kp) {
+    constexpr int kPath = !COLS ? kPathTeams : (DVX > 0 ? kPathColumns : kPathLong);
     extern __shared__ __align__(16) unsigned char smem[];
     BlockHdr *hdr = reinterpret_cast<BlockHdr *>(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1653,15 +1669,15 @@ __global__ void __launch_bounds__(COLS ? kColumnThreads : 512, MINB) bpsf_persis
             const StreamDev &d = kp.streams[sid];
             if (tid == 0)
                 *reinterpret_cast<TeamOffsets *>(smem + kBlockHeaderBytes + kStreamBytes) =
-                    team_offsets(d.S, d.code.M, d.code.N, d.code.P, d.code.Ws, 0, FB, true);
+                    team_offsets(d.S, d.code.M, d.code.N, d.code.P, d.code.Ws, 0, FB, kPath);
             __syncthreads();
         }
         const StreamDev &sd = COLS ? *reinterpret_cast<const StreamDev *>(smem + kBlockHeaderBytes) : kp.streams[sid];
         const CodeDev &cd = sd.code;
         const int S = sd.S, W = sd.W, teams = sd.teams;
-        const LayoutOffsets lo = layout_offsets(cd.M, cd.N, DVS, cd.P, COLS);
+        const LayoutOffsets lo = layout_offsets(cd.M, cd.N, DVS, cd.P, kPath);
         unsigned char *lay = smem + kBlockHeaderBytes + (COLS ? kDescriptorBytes : 0);
-        if (sid != cur && !COLS) {
+        if (sid != cur && kPath != kPathColumns) {
             uint8_t *rd = lay + lo.row_deg;
             uint16_t *vp = reinterpret_cast<uint16_t *>(lay + lo.vpos);
             float *lc = reinterpret_cast<float *>(lay + lo.lch);
@@ -1669,7 +1685,7 @@ __global__ void __launch_bounds__(COLS ? kColumnThreads : 512, MINB) bpsf_persis
             for (int k = tid; k < cd.M; k += blockDim.x) rd[k] = cd.row_deg[k];
             for (int k = tid; k < cd.N * DVS; k += blockDim.x) vp[k] = cd.vpos[k];
             for (int k = tid; k < cd.N; k += blockDim.x) lc[k] = cd.lch[k];
-            for (int k = tid; k < cd.P; k += blockDim.x) lp[k] = cd.lch_pos[k];
+            for (int k = tid; kPath == kPathTeams && k < cd.P; k += blockDim.x) lp[k] = cd.lch_pos[k];
         }
         cur = sid;
         // Every slot starts empty; teams start idle.
@@ -1716,7 +1732,7 @@ __global__ void __launch_bounds__(COLS ? kColumnThreads : 512, MINB) bpsf_persis
         L.lch = reinterpret_cast<const float *>(lay + lo.lch);
         L.lch_pos = reinterpret_cast<const float *>(lay + lo.lch_pos);
         if (warp == 0) {
-            manager_loop<DEBUG>(sd, L, team_base, to.total, to, teams, S, qbase, Q, hdr, lane, kp.wait_ns);
+            manager_loop<DEBUG, COLS>(sd, L, team_base, to.total, to, teams, S, qbase, Q, hdr, lane, kp.wait_ns);
         } else {
             const int team = (warp - 1) / W;
             if (team < teams) {
@@ -1724,10 +1740,12 @@ __global__ void __launch_bounds__(COLS ? kColumnThreads : 512, MINB) bpsf_persis
                 const int ttid = tid - 32 - team * W * 32;
                 if constexpr (COLS) {
                     const int tb = keep((int)(team_base - smem) + team * to.total);
-                    if (S == 4)
-                        column_loop<DC, DVX, DVS, 4, DEBUG, FB>(sd, to, hdr, tb, W, ttid, 1 + team);
+                    if constexpr (DVX == 0)
+                        column_loop<DC, 3, DVS, kLongSlots, true, DEBUG, FB>(sd, to, hdr, L, tb, W, ttid, 1 + team);
+                    else if (S == 4)
+                        column_loop<DC, DVX, DVS, 4, false, DEBUG, FB>(sd, to, hdr, L, tb, W, ttid, 1 + team);
                     else
-                        column_loop<DC, DVX, DVS, 1, DEBUG, FB>(sd, to, hdr, tb, W, ttid, 1 + team);
+                        column_loop<DC, DVX, DVS, 1, false, DEBUG, FB>(sd, to, hdr, L, tb, W, ttid, 1 + team);
                 } else if (MIX && cd.regular && cd.DC == 6 && cd.dv_max == 3)
                     team_loop<6, DVS, 3, DEBUG, MINB, LAY, FB>(sd, L, T, hdr, S, W, ttid, 1 + team, kp.wait_ns);
                 else

@@ -68,6 +68,17 @@ def test_column_path(m, alpha, max_iter):
     run(rng, regular(rng, m), 4, False, alpha, max_iter)
 
 
+# Lanes that loop over a long code's columns and rows: fewer, exactly as many and
+# more of them than lanes; column degrees 0 to 3, row degrees 2 to 8.
+@pytest.mark.parametrize("m,n,dc,alpha", [(480, 864, 8, 0.625), (432, 865, 8, 0.0), (700, 1800, 7, 0.625),
+                                          (864, 1728, 8, 0.0)])
+def test_long_codes(m, n, dc, alpha):
+    rng = np.random.default_rng(m)
+    h = irregular(rng, m, n, dc, 3)
+    assert h.sum() > 2048
+    run(rng, h, 1, False, alpha)
+
+
 @pytest.mark.parametrize("select", [B.BPSF_SELECT_MIN_WEIGHT, B.BPSF_SELECT_FIRST])
 @pytest.mark.parametrize("shots", [1, 7, 8, 500])  # one and four slots per team
 def test_column_path_equals_teams(shots, select):
