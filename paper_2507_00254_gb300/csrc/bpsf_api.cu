@@ -710,6 +710,9 @@ extern "C" bpsf_status bpsf_create(bpsf_ctx **out, int32_t M, int32_t N, int64_t
     cd.n_trials = c->n_trials;
     cd.select = p.select;
     cd.alpha = p.alpha;
+    cd.lch0 = lch[0];
+    cd.uniform = 1;
+    for (int i = 1; i < N; ++i) cd.uniform = cd.uniform && lch[i] == lch[0];
     cd.row_deg = (const uint8_t *)(base + off[0]);
     cd.vchk = (const uint16_t *)(base + off[1]);
     cd.lch = (const float *)(base + off[2]);

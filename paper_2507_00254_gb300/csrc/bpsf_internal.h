@@ -60,6 +60,8 @@ struct CodeDev {
     int vstride;                 // entries per column in vpos / vchk (>= dv_max)
     int max_iter, short_iter, w, n_trials, select;
     float alpha;
+    int uniform;                 // 1: every channel LLR is lch0
+    float lch0;
     const uint8_t *row_deg;      // M, ones per row
     const uint16_t *vpos;        // N x vstride, message positions (0xffff padding), active layout
     const uint16_t *vchk;        // N x vstride, check indices
@@ -269,6 +271,7 @@ struct TeamCtl {
     unsigned long long iters;  // iterations run by this team (all slots)
     unsigned long long cap;    // team iterations with a running slot, times S
     int flushed;               // column path: team iterations already in cap
+    unsigned fresh;            // slots whose run starts with the next iteration (as run_mask)
 };
 static_assert(sizeof(TeamCtl) <= 64, "team control block fits its 64 bytes");
 

@@ -65,6 +65,11 @@ __device__ __forceinline__ int keep(int x) {
     asm volatile("" : "+r"(x));
     return x;
 }
+template <typename T>
+__device__ __forceinline__ const T *keep(const T *p) {
+    asm volatile("" : "+l"(p));
+    return p;
+}
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
@@ -215,6 +220,29 @@ BPSF_VOP(vadd, "add.rn.f32x2", __fadd_rn)
 BPSF_VOP(vsub, "sub.rn.f32x2", __fsub_rn)
 #undef BPSF_VOP
 
+// a * b + d, slot by slot, rounded once.
+template <int V>
+__device__ __forceinline__ void vfma(float (&o)[V], const float (&a)[V], const float (&b)[V], const float (&d)[V]) {
+    if (V == 1) {
+        o[0] = __fmaf_rn(a[0], b[0], d[0]);
+    } else {
+#pragma unroll
+        for (int c = 0; c + 1 < V; c += 2)
+            asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
+                "fma.rn.f32x2 x, x, y, z;\n\tmov.b64 {%0, %1}, x;\n\t}"
+                : "=f"(o[c]), "=f"(o[c + 1])
+                : "f"(a[c]), "f"(a[c + 1]), "f"(b[c]), "f"(b[c + 1]), "f"(d[c]), "f"(d[c + 1]));
+    }
+}
+
+// What the phases of the team path read of the code in every iteration, in registers.
+struct Hot {
+    int M, N, Mp;
+    const uint16_t *vchk;
+    bool uniform;  // all channel LLRs are lch0
+    float lch0;
+};
+
 // min(|a|, |b|) with the product of the two signs: one instruction.
 __device__ __forceinline__ float min_sign(float a, float b) {
     float o;
@@ -304,9 +332,13 @@ __device__ __forceinline__ void row_outputs(float (&x)[DC][V], const float (&see
 }
 
 // One row for V adjacent slots.  tauv = j*(S/V) + q; MQ: rank stride in V-slot groups.
+// The factors' inputs are alpha q + beta.  A running slot has its damping factor
+// and -0 (which changes nothing).  In the first iteration of a run whose channel
+// LLRs are all the same, alpha is 0 and beta the damped LLR: its messages need
+// not be set up, which took as much shared-memory traffic as two iterations.
 template <int DC, bool REG, int V>
 __device__ __forceinline__ void c_row(const LayoutMem &L, const TeamMem &T, int MQ, int lgQ, int tauv,
-                                      const float (&alpha)[V]) {
+                                      const float (&alpha)[V], const float (&beta)[V]) {
     typedef typename VecF<V>::T VT;
     VT *pv = reinterpret_cast<VT *>(T.m) + tauv;
     const int deg = REG ? DC : (int)L.row_deg[tauv >> lgQ];
@@ -316,7 +348,7 @@ __device__ __forceinline__ void c_row(const LayoutMem &L, const TeamMem &T, int 
     for (int k = 0; k < DC; ++k)
         if (REG || k < deg) {
             vload<V>(x[k], pv + k * MQ);
-            vmul<V>(x[k], x[k], alpha);
+            vfma<V>(x[k], x[k], alpha, beta);
         } else {
 #pragma unroll
             for (int c = 0; c < V; ++c) x[k][c] = __int_as_float(0x7f800000);
@@ -329,12 +361,12 @@ __device__ __forceinline__ void c_row(const LayoutMem &L, const TeamMem &T, int 
 }
 
 template <int DC, bool REG, int V>
-__device__ __forceinline__ void c_phase(const CodeDev &cd, const LayoutMem &L, const TeamMem &T, int lgS,
-                                        const float (&alpha)[V], int tid, int nthreads) {
+__device__ __forceinline__ void c_phase(const Hot &h, const LayoutMem &L, const TeamMem &T, int lgS,
+                                        const float (&alpha)[V], const float (&beta)[V], int tid, int nthreads) {
     const int lgQ = lgS - (V == 4 ? 2 : V - 1);
-    const int MQ = cd.Mp << lgQ;  // rank stride of the active layout, in V-slot groups
-    const int nt = cd.M << lgQ;   // row tasks (rows M..Mp-1 of the stride are padding)
-    for (int tauv = tid; tauv < nt; tauv += nthreads) c_row<DC, REG, V>(L, T, MQ, lgQ, tauv, alpha);
+    const int MQ = h.Mp << lgQ;  // rank stride of the active layout, in V-slot groups
+    const int nt = h.M << lgQ;   // row tasks (rows M..Mp-1 of the stride are padding)
+    for (int tauv = tid; tauv < nt; tauv += nthreads) c_row<DC, REG, V>(L, T, MQ, lgQ, tauv, alpha, beta);
 }
 
 // ---------------------------------------------------------------------------
@@ -428,9 +460,9 @@ template <> struct FlipPack<1, 4> {
 // The residual syndrome s xor H e toggles at the checks of column i for the
 // slots in bm (bit c*S + s of the team's residual-syndrome words).
 template <int DVS, int DVX>
-__device__ __forceinline__ void toggle_residual(const CodeDev &cd, const TeamMem &T, int lgS, int s0, int i,
+__device__ __forceinline__ void toggle_residual(const uint16_t *vchk, const TeamMem &T, int lgS, int s0, int i,
                                                 unsigned bm) {
-    const uint16_t *vc = cd.vchk + i * DVS;
+    const uint16_t *vc = vchk + i * DVS;
     uint16_t chk[DVS];
     if (DVS == 4) {
         const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(vc));
@@ -451,14 +483,13 @@ __device__ __forceinline__ void toggle_residual(const CodeDev &cd, const TeamMem
     }
 }
 
-template <int DVS, int DVX, bool DEBUG, int V, int FB>
-__device__ __forceinline__ void v_phase(const StreamDev &sd, const LayoutMem &L, const TeamMem &T, int lgS,
+template <int DVS, int DVX, bool DEBUG, int V, int FB, bool UNI>
+__device__ __forceinline__ void v_phase(const StreamDev &sd, const Hot &h, const LayoutMem &L, const TeamMem &T, int lgS,
                                         unsigned onm, unsigned initm, int tid, int nthreads) {
     typedef typename VecF<V>::T VT;
     typedef FlipPack<FB, V> FP;
-    const CodeDev &cd = sd.code;
     const int lgQ = lgS - (V == 4 ? 2 : V - 1);
-    const int total = cd.N << lgQ;
+    const int total = h.N << lgQ;
     const int q = tid & ((1 << lgQ) - 1);
     const int s0 = V * q;
     VT *mv = reinterpret_cast<VT *>(T.m) + q;
@@ -481,7 +512,7 @@ __device__ __forceinline__ void v_phase(const StreamDev &sd, const LayoutMem &L,
         }
         float lc[V];
         {
-            const float l = L.lch[i];
+            const float l = UNI && h.uniform ? h.lch0 : L.lch[i];
 #pragma unroll
             for (int c = 0; c < V; ++c) lc[c] = l;
         }
@@ -518,12 +549,12 @@ __device__ __forceinline__ void v_phase(const StreamDev &sd, const LayoutMem &L,
 #pragma unroll
             for (int c = 0; c < V; ++c)
                 if (((onm >> c) & 1u) && ((initm >> (s0 + c)) & 1u))
-                    sd.dbg.lout[T.st[s0 + c].shot * cd.N + i] = __fsub_rn(0.f, nl[c]);
+                    sd.dbg.lout[T.st[s0 + c].shot * h.N + i] = __fsub_rn(0.f, nl[c]);
         }
         const typename FP::D d = FP::diff(nl, fw, on);
         if (FP::any(d)) {
             fv[tauv] = FP::bump(fw, d);
-            toggle_residual<DVS, DVX>(cd, T, lgS, s0, i, FP::slots(d));
+            toggle_residual<DVS, DVX>(h.vchk, T, lgS, s0, i, FP::slots(d));
         }
     }
 }
@@ -612,7 +643,7 @@ __device__ __forceinline__ void layered_iteration(const StreamDev &sd, const Lay
         const typename FP::D d = FP::diff(nl, fw, on);
         if (FP::any(d)) {
             fv[tauv] = FP::bump(fw, d);
-            toggle_residual<DVS, DVX>(cd, T, lgS, s0, i, FP::slots(d));
+            toggle_residual<DVS, DVX>(cd.vchk, T, lgS, s0, i, FP::slots(d));
         }
     }
 }
@@ -756,7 +787,7 @@ __device__ __forceinline__ void team_pack(const StreamDev &sd, const TeamMem &T,
 // residual-syndrome words (atomic toggles of the bits that differ: lanes
 // share words), its V2C messages set to the channel LLRs (the first C phase
 // reads l_ch on every edge), its decision and flip-count words zeroed.
-template <int FB>
+template <int FB, bool UNI>
 __device__ __forceinline__ void team_install(const StreamDev &sd, const LayoutMem &L, const TeamMem &T, int S, int s,
                                              int lane) {
     const CodeDev &cd = sd.code;
@@ -775,7 +806,7 @@ __device__ __forceinline__ void team_install(const StreamDev &sd, const LayoutMe
         // Layered schedule: C2V messages start at zero, the posterior at l_ch.
         for (int k = lane; k < cd.P; k += 32) T.m[k * S + s] = 0.f;
         for (int i = lane; i < cd.N; i += 32) T.post[i * S + s] = L.lch[i];
-    } else {
+    } else if (!UNI || !cd.uniform) {  // else see c_row
         for (int k = lane; k < cd.P; k += 32) T.m[k * S + s] = L.lch_pos[k];
     }
     for (int i = lane; i < cd.N; i += 32) flipw<FB>(T)[i * S + s] = 0;
@@ -793,7 +824,7 @@ __device__ __forceinline__ void team_install(const StreamDev &sd, const LayoutMe
     __syncwarp();
 }
 
-template <bool DEBUG, int FB>
+template <bool DEBUG, int FB, bool UNI>
 __device__ __forceinline__ void team_service(const StreamDev &sd, const LayoutMem &L, const TeamMem &T, int S, int lgS,
                                              int lane, unsigned long long wait_ns) {
     const int stv = lane < S ? *vstate(&T.st[lane]) : kSlotRunning;
@@ -819,7 +850,7 @@ __device__ __forceinline__ void team_service(const StreamDev &sd, const LayoutMe
         const int s = __ffs(im) - 1;
         im &= im - 1u;
         const int kind = reinterpret_cast<const QEntry *>(T.ib + s * T.ibstride)->kind;
-        if (kind != 0) team_install<FB>(sd, L, T, S, s, lane);
+        if (kind != 0) team_install<FB, UNI>(sd, L, T, S, s, lane);
         __syncwarp();
         if (lane == 0) {
             // RUNNING before the inbox reads empty: the manager's exit test
@@ -853,7 +884,7 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
     const int lane = tid & 31, wt = tid >> 5, nthreads = 32 * W;
     const CodeDev &cd = sd.code;
     const int lgS = __ffs(S) - 1;
-    const int n_rwords = ((cd.M << lgS) + 31) >> 5;  // residual-syndrome words of the team
+    const int n_rwords = MINB == 1 ? keep(((cd.M << lgS) + 31) >> 5) : ((cd.M << lgS) + 31) >> 5;  // residual-syndrome words of the team
     const unsigned full = S >= 32 ? 0xffffffffu : ((1u << S) - 1u);
     constexpr bool kVec = DC <= 16;  // the widest rows keep one slot per lane (registers)
     // Four slots per lane: exact-degree rows with the full register budget (one block).
@@ -861,6 +892,12 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
     // Layered schedule: vector lanes in the full-register instances only.
     constexpr bool kLayV2 = LAY && kVec && MINB == 1 && DC <= 6, kLayV4 = kLayV2 && kVec4;
     const bool lay = LAY && cd.layered;
+    // The 64-register instance has no registers for this: it spilled, and 200 000
+    // [[72]] shots took 6.6 instead of 5.7 ms.
+    Hot h = {cd.M, cd.N, cd.Mp, cd.vchk, false, 0.f};
+    if (MINB == 1) h = {keep(h.M), keep(h.N), keep(h.Mp), keep(h.vchk), keep(cd.uniform) != 0 && !lay, cd.lch0};
+    const float alpha0 = cd.alpha;
+    unsigned fresh = 0u;  // slots in the first iteration of their run
     // Slots per lane in the phases (vs) and the lane's first slot (s0).
     const int vs = lay ? ((kLayV4 && S >= 4) ? 4 : ((kLayV2 && S >= 2) ? 2 : 1))
                        : ((kVec4 && S >= 4) ? 4 : ((kVec && S >= 2) ? 2 : 1));
@@ -900,13 +937,14 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
                     n_iters = 0;
                     tt_flush = tt;
                 }
-                team_service<DEBUG, FB>(sd, L, T, S, lgS, lane, wait_ns);
+                team_service<DEBUG, FB, MINB == 1>(sd, L, T, S, lgS, lane, wait_ns);
                 SlotState *ss = &T.st[lane < S ? lane : 0];
                 const int stv = lane < S ? *vstate(ss) : kSlotEmpty;
                 const bool r = stv == kSlotRunning;
                 __threadfence_block();
                 const unsigned rm = __ballot_sync(FULLMASK, r);
                 const unsigned im = __ballot_sync(FULLMASK, r && ss->kind == 1);
+                const unsigned fm = __ballot_sync(FULLMASK, r && ss->start < 0);
                 // A run installed at this service starts with the next iteration.
                 if (r && ss->start < 0) ss->start = tt;
                 int ex = 0;
@@ -945,12 +983,14 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
                 if (lane == 0) {
                     T.ctl->run_mask = rm;
                     T.ctl->init_mask = im;
+                    T.ctl->fresh = fm;
                     T.ctl->exit = ex;
                 }
             }
             team_sync(W, bar_id);
             run = T.ctl->run_mask;
             initm = T.ctl->init_mask;
+            if (MINB == 1) fresh = T.ctl->fresh;
             const int ex = T.ctl->exit;
             if (ex) break;
             if (run == 0u) continue;
@@ -970,10 +1010,15 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
         }
         // Damping of iteration it = tt - start + 1 of each of the lane's slots
         // (the start is read only under adaptive damping).
-        float al[4];
+        float al[4], be[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            al[c] = adaptive && c < vs ? damping(cd, tt - T.st[s0 + c].start + 1) : cd.alpha;
+        for (int c = 0; c < 4; ++c) {
+            al[c] = adaptive && c < vs ? damping(cd, tt - T.st[s0 + c].start + 1) : alpha0;
+            const bool f = MINB == 1 && h.uniform && ((fresh >> (s0 + c)) & 1u) && c < vs;
+            be[c] = f ? __fmul_rn(damping(cd, 1), h.lch0) : -0.0f;
+            al[c] = f ? 0.f : al[c];
+        }
+        fresh = 0u;
         const unsigned onm = (run >> s0) & ((1u << vs) - 1u);  // the lane's running slots
         if (lay) {
             if (kLayV4 && vs == 4) {
@@ -986,19 +1031,19 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
                 layered_iteration<DC, DVS, DVX, DEBUG, 1, FB>(sd, L, T, lgS, onm, a1, initm, tid, nthreads, W, bar_id);
             }
         } else if (kVec4 && vs == 4) {
-            if (onm) c_phase<DC, (DVX > 0), 4>(cd, L, T, lgS, al, tid, nthreads);
+            if (onm) c_phase<DC, (DVX > 0), 4>(h, L, T, lgS, al, be, tid, nthreads);
             team_sync(W, bar_id);
-            if (onm) v_phase<DVS, DVX, DEBUG, 4, FB>(sd, L, T, lgS, onm, initm, tid, nthreads);
+            if (onm) v_phase<DVS, DVX, DEBUG, 4, FB, MINB == 1>(sd, h, L, T, lgS, onm, initm, tid, nthreads);
         } else if (kVec && vs == 2) {
-            const float a2[2] = {al[0], al[1]};
-            if (onm) c_phase<DC, (DVX > 0), 2>(cd, L, T, lgS, a2, tid, nthreads);
+            const float a2[2] = {al[0], al[1]}, b2[2] = {be[0], be[1]};
+            if (onm) c_phase<DC, (DVX > 0), 2>(h, L, T, lgS, a2, b2, tid, nthreads);
             team_sync(W, bar_id);
-            if (onm) v_phase<DVS, DVX, DEBUG, 2, FB>(sd, L, T, lgS, onm, initm, tid, nthreads);
+            if (onm) v_phase<DVS, DVX, DEBUG, 2, FB, MINB == 1>(sd, h, L, T, lgS, onm, initm, tid, nthreads);
         } else {
-            const float a1[1] = {al[0]};
-            if (onm) c_phase<DC, (DVX > 0), 1>(cd, L, T, lgS, a1, tid, nthreads);
+            const float a1[1] = {al[0]}, b1[1] = {be[0]};
+            if (onm) c_phase<DC, (DVX > 0), 1>(h, L, T, lgS, a1, b1, tid, nthreads);
             team_sync(W, bar_id);
-            if (onm) v_phase<DVS, DVX, DEBUG, 1, FB>(sd, L, T, lgS, onm, initm, tid, nthreads);
+            if (onm) v_phase<DVS, DVX, DEBUG, 1, FB, MINB == 1>(sd, h, L, T, lgS, onm, initm, tid, nthreads);
         }
         team_sync(W, bar_id);
         // Decision, in every warp: slot s owns bits s, s + S, s + 2S, ... of
@@ -1687,6 +1732,7 @@ __global__ void __launch_bounds__(COLS ? (DVX > 0 ? kColumnThreads : kLongThread
             for (int k = tid; k < cd.N; k += blockDim.x) lc[k] = cd.lch[k];
             for (int k = tid; kPath == kPathTeams && k < cd.P; k += blockDim.x) lp[k] = cd.lch_pos[k];
         }
+        const bool fill = sid != cur;
         cur = sid;
         // Every slot starts empty; teams start idle.
         TeamOffsets to_reg;
@@ -1719,6 +1765,14 @@ __global__ void __launch_bounds__(COLS ? (DVX > 0 ? kColumnThreads : kLongThread
                 const int t = k / sw, w = k - t * sw;
                 reinterpret_cast<uint32_t *>(team_base + t * to.total + to.syn)[w] = 0u;
             }
+        }
+        // Messages that no install sets up (uniform channel LLRs) start finite: the
+        // first iteration multiplies them by zero.
+        if (kPath == kPathTeams && cd.uniform && !cd.layered && fill) {
+            const int words = to.m + 4 * S * cd.P;
+            for (int t = 0; t < teams; ++t)
+                for (int k = to.m / 4 + tid; k < words / 4; k += blockDim.x)
+                    reinterpret_cast<uint32_t *>(team_base + t * to.total)[k] = 0u;
         }
         if (tid == 0) {
             hdr->exit = 0;
