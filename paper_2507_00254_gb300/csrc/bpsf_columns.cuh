@@ -152,7 +152,7 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                 for (int k = 0; k < DC; ++k)
                     if (!LONG || k < deg) vstore<CV>(reinterpret_cast<CT *>(row + k * mstride), x[k]);
             };
-            if (LONG) {
+            if constexpr (LONG) {
 #pragma unroll 1
                 for (int task = tid; task < CG * M; task += nth) row_part(task);
                 if (4 * lane < nw) w4 = *reinterpret_cast<const uint4 *>(smem + o_mism + 16 * lane);
@@ -329,9 +329,10 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                             // The stored C2V messages carry the opposite sign.
                             const int j = tid / CG;
                             const unsigned b = (src[j >> 5] >> (j & 31)) & 1u;
-#pragma unroll
-                            for (int h = 0; h < CV; ++h)
-                                if (c % CV == h) seed[h] = __uint_as_float((b ? 0u : 0x80000000u) | 0x71800000u);
+                            const float v = __uint_as_float((b ? 0u : 0x80000000u) | 0x71800000u);
+                            const bool last = CV == 1 || (c & 1);  // selects: an index would put the array in memory
+                            seed[0] = CV > 1 && last ? seed[0] : v;
+                            seed[CV - 1] = last ? v : seed[CV - 1];
                         }
                         flip_clear<FB, V>(fw, c);
                     } else {
@@ -351,11 +352,13 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                         for (int i = tid; i < N; i += nth) flipw<FB>(T)[(i << lgS) + c] = 0;
                     }
                     if (c / CV == tid % CG) {
-#pragma unroll
-                        for (int h = 0; h < CV; ++h)
-                            if (adaptive && c % CV == h) al[h] = 0.5f;
+                        const bool last = CV == 1 || (c & 1);
+                        al[0] = !adaptive || (CV > 1 && last) ? al[0] : 0.5f;
+                        al[CV - 1] = adaptive && last ? 0.5f : al[CV - 1];
                     }
                     // The row's first C2V messages, by its syndrome bit.
+                    const bool same = cd.uniform != 0;
+                    const float first = fminf(__fmul_rn(adaptive ? 0.5f : cd.alpha, cd.lch0), kMagClamp);
                     for (int j = tid; j < M; j += nth) {
                         const unsigned flip = ((src[j >> 5] >> (j & 31)) & 1u) ? 0u : 0x80000000u;
                         const int dj = LONG ? (int)L.row_deg[j] : DC;
@@ -364,7 +367,7 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                         for (int k = 0; k < DC; ++k)
                             if (!LONG || k < dj)
                                 msg[k * (mstride >> 2)] =
-                                    __uint_as_float(__float_as_uint(__ldg(cd.c2v0 + k * cd.Mp + j)) ^ flip);
+                                    __uint_as_float(__float_as_uint(same ? first : __ldg(cd.c2v0 + k * cd.Mp + j)) ^ flip);
                     }
                     if (sw) {
                         for (int w = lane; !LONG && w < cd.Ws; w += 32) T.syn[c * cd.Ws + w] = src[w];
@@ -455,7 +458,7 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                 }
             }
         };
-        if (!LONG) {
+        if constexpr (!LONG) {
             if (tid < N) column(tid, mcol, lc, fw);
         } else {
             typename FP::U *fl = reinterpret_cast<typename FP::U *>(smem + o_flips);
