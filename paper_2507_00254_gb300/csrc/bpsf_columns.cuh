@@ -254,9 +254,10 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                 for (unsigned m = pk; m; m &= m - 1u) {
                     const int c = __ffs(m) - 1;
                     const bool counts = ((initm & ~pconv) >> c) & 1u;
-                    // A converged initial run's decision is the shot's result.
+                    // A long code's converged initial run: its decision goes out at once (the
+                    // manager's one lane would write 81 words).
                     uint32_t *words = T.ebits + c * cd.Wn;
-                    if ((initm & pconv) >> c & 1u) words = sd.job.corr + row_of(sd, T.st[c].shot) * sd.job.corr_stride;
+                    if (LONG && ((initm & pconv) >> c & 1u)) words = sd.job.corr + row_of(sd, T.st[c].shot) * sd.job.corr_stride;
 #pragma unroll 2
                     for (int i0 = tid - lane; i0 < N; i0 += nth) {
                         const int i = i0 + lane;
@@ -356,7 +357,7 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                         al[0] = !adaptive || (CV > 1 && last) ? al[0] : 0.5f;
                         al[CV - 1] = adaptive && last ? 0.5f : al[CV - 1];
                     }
-                    // The row's first C2V messages, by its syndrome bit.
+                    // The rows' first C2V messages, by their syndrome bits.
                     const bool same = cd.uniform != 0;
                     const float first = fminf(__fmul_rn(adaptive ? 0.5f : cd.alpha, cd.lch0), kMagClamp);
                     for (int j = tid; j < M; j += nth) {

@@ -1166,9 +1166,9 @@ __device__ __forceinline__ bool trial_cannot_win(const StreamDev &sd, long long 
 }
 
 // Lane-parallel write-out of outboxes that need no warp cooperation:
-// converged or uncorrectable initial runs, and trial runs.  (COLS: a converged
+// converged or uncorrectable initial runs, and trial runs.  (LONG: a converged
 // initial run's words are out already.)
-template <bool DEBUG, bool COLS>
+template <bool DEBUG, bool LONG>
 __device__ __forceinline__ void finalize_simple(const StreamDev &sd, TeamMem T, int s, MgrState &mg) {
     const CodeDev &cd = sd.code;
     const JobDev &job = sd.job;
@@ -1184,7 +1184,7 @@ __device__ __forceinline__ void finalize_simple(const StreamDev &sd, TeamMem T, 
         // output (written by its team before it published the trials).
         if (!conv && cd.w > 0) return;
         uint32_t *out = job.corr + row * job.corr_stride;
-        if (!COLS || !conv)
+        if (!LONG || !conv)
             for (int w = 0; w < Wn; ++w) out[w] = slot_word(T.ebits, Wn, s, w);
         job.conv[row] = conv ? 1 : 0;
         job.iters[row] = (int16_t)(conv ? iter : cd.max_iter);
@@ -1449,7 +1449,7 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
     return got_any;
 }
 
-template <bool DEBUG, bool COLS>
+template <bool DEBUG, bool LONG>
 __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned char *team_base, int team_bytes,
                              const TeamOffsets &to, int teams, int S, unsigned char *qbase, int Q, BlockHdr *hdr,
                              int lane, unsigned long long wait_ns) {
@@ -1483,7 +1483,7 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
                 if (T.st[s].cancel != key && trial_cannot_win(sd, T.st[s].rec, kidx))
                     *reinterpret_cast<volatile long long *>(&T.st[s].cancel) = key;
             }
-            if (fin) finalize_simple<DEBUG, COLS>(sd, T, s, mg);
+            if (fin) finalize_simple<DEBUG, LONG>(sd, T, s, mg);
             __syncwarp();
             if (fin) {
                 __threadfence_block();
@@ -1786,7 +1786,7 @@ __global__ void __launch_bounds__(COLS ? (DVX > 0 ? kColumnThreads : kLongThread
         L.lch = reinterpret_cast<const float *>(lay + lo.lch);
         L.lch_pos = reinterpret_cast<const float *>(lay + lo.lch_pos);
         if (warp == 0) {
-            manager_loop<DEBUG, COLS>(sd, L, team_base, to.total, to, teams, S, qbase, Q, hdr, lane, kp.wait_ns);
+            manager_loop<DEBUG, kPath == kPathLong>(sd, L, team_base, to.total, to, teams, S, qbase, Q, hdr, lane, kp.wait_ns);
         } else {
             const int team = (warp - 1) / W;
             if (team < teams) {
