@@ -64,8 +64,10 @@ static size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
 static void free_workspace(bpsf_ctx *c) {
     if (c->d_rec) {
-        // The counters of the last launch stay readable (bpsf_sync).
+        // The counters of the last launch stay readable (bpsf_sync); it may still be
+        // running, and a copy does not wait for other streams as cudaFree does.
         if (c->d_ctr_last == c->w_ctr) {
+            cudaDeviceSynchronize();
             cudaMemcpy(c->d_ctr, c->w_ctr, kCounterBytes, cudaMemcpyDeviceToDevice);
             c->d_ctr_last = c->d_ctr;
         }

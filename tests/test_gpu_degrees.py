@@ -96,6 +96,24 @@ def test_column_path_equals_teams(shots, select):
         assert all(work[k] == v for k, v in d.last_work().items() if k != "slot_capacity")
 
 
+@pytest.mark.parametrize("shots", [300, 20001])
+def test_counters_outlive_the_workspace(shots):
+    """A new trial list frees the workspace of a decode that may still be running."""
+    c = codes.bb("bb144")
+    d = B.Decoder(c.ptr, c.idx, c.M, c.N, np.full(c.N, 0.07), B.Params(max_iter=60, w=6, short_iter=20))
+    rng = np.random.default_rng(shots)
+    e = (rng.random((shots, c.N)) < 0.08).astype(np.uint8)
+    synd = d.syndrome(torch.from_numpy(harness.pack_rows(e).view(np.int32)).cuda())
+    d.decode(synd)
+    want = d.last_work()
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    d.decode(synd, stream=stream, sync=False)
+    d.set_trials([])
+    B.bpsf_sync(d.handle, stream.cuda_stream)
+    assert all(d.last_work()[k] == v for k, v in want.items() if k != "slot_capacity")
+
+
 def run(rng, h, slots, layered, alpha, max_iter=40, blocks=0):
     m, n = h.shape
     idx = np.concatenate([np.nonzero(r)[0] for r in h])
