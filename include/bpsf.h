@@ -257,8 +257,10 @@ bpsf_status bpsf_sync(bpsf_ctx *ctx, void *stream);
  * Small batches (up to about 1.5 * 10^6 shots times columns in a launch, for
  * example 10^4 shots of [[144,12,12]]) of codes of row weight 6 and column
  * weight 3 without the layered schedule run with a lane per column instead, on
- * a shape of their own, unless blocks_per_sm is given.  Results do not depend
- * on it.
+ * a shape of their own, unless blocks_per_sm is given.  So do batches of any
+ * size of codes with ten ones in every row and five in every column, and of
+ * long codes (more than 2048 ones in H, at most eight in a row and three in a
+ * column, not all rows with six and columns with three).  Results do not depend on it.
  */
 typedef struct {
     int32_t warps_per_team;  /* 1, 2, 4 or 8 */

@@ -180,10 +180,16 @@ constexpr long long kColumnShots = 1500000;
 // any batch.  In teams of four warps with a slot each, three warps waited while
 // one packed and installed 2592 columns.  10^5 shots of the 12-round
 // phenomenological [[144]] at p = q = 0.004: 7.6 ms in such teams, 4.6 with 27
-// warps on four slots, 4.7 with 19 warps, 5.7 with 27 on two slots.
-static bool plan_long(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, bpsf_plan *out, int *variant, int *B,
-                      int *smem, int Q) {
+// warps on four slots, 4.7 with 19 warps, 5.7 with 27 on two slots.  Exact (6, 3)
+// codes have their own team loop, which wins where it does against the other
+// column path: 784 columns at p = 0.05, 1000 shots 1.01 against 0.97 ms, 20 000
+// 15.7 / 11.7; at p = 0.01 0.32 / 0.30 and 0.86 / 0.62.
+static bool plan_long(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, const long long *shots, bool exact,
+                      bpsf_plan *out, int *variant, int *B, int *smem, int Q) {
     int bytes = 0;
+    long long work = 0;
+    for (int k = 0; k < n_codes; ++k) work += std::min(shots[k], kColumnShots) * codes[k]->N;
+    if (exact && work > kColumnShots) return false;
     for (int k = 0; k < n_codes; ++k) {
         const bpsf_ctx *c = codes[k];
         if (c->nnz <= kMaxShardNnz || c->dc_max > 8 || c->dv_max > 3 || c->vstride != 4) return false;
@@ -313,7 +319,7 @@ bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tunin
         if (any_exact) variant = kernel_variant_mixed(variant);
     }
     long long grid_max = 1ll << 30;
-    if (shots && plan_long(codes, n_codes, tunes, out, &variant, &B, &smem, Q)) {
+    if (shots && plan_long(codes, n_codes, tunes, shots, all_regular && dc == 6 && dv == 3, out, &variant, &B, &smem, Q)) {
     } else if (shots && all_regular && !layered)
         plan_columns(codes, n_codes, tunes, shots, dc, dv, out, &variant, &B, &smem, &grid_max, Q);
     bpsf_status st = bpsf_ensure_kernel_attrs(variant, c0->smem_optin);

@@ -79,6 +79,22 @@ def test_long_codes(m, n, dc, alpha):
     run(rng, h, 1, False, alpha)
 
 
+# Long codes of six ones per row and three per column: the lanes' loop up to
+# 1.5e6 shots times columns (2192 shots here), teams beyond.
+@pytest.mark.parametrize("alpha", [0.625, 0.0])
+def test_long_exact_codes_by_batch(alpha):
+    rng = np.random.default_rng(342)
+    h = regular(rng, 342)
+    m, n = h.shape
+    idx = np.concatenate([np.nonzero(r)[0] for r in h])
+    ptr = np.concatenate([[0], np.cumsum(h.sum(axis=1))])
+    d = B.Decoder(ptr, idx, m, n, np.full(n, 0.03), B.Params(max_iter=40, alpha=alpha, w=4, short_iter=9))
+    e = (rng.random((2193, n)) < 0.03).astype(np.uint8)
+    synd = d.syndrome(torch.from_numpy(harness.pack_rows(e).view(np.int32)).cuda())
+    few, many = d.decode(synd[:2192]), d.decode(synd)
+    assert all(torch.equal(few[k], many[k][:2192]) for k in few)
+
+
 @pytest.mark.parametrize("select", [B.BPSF_SELECT_MIN_WEIGHT, B.BPSF_SELECT_FIRST])
 @pytest.mark.parametrize("shots", [1, 7, 8, 500])  # one and four slots per team
 def test_column_path_equals_teams(shots, select):
