@@ -36,10 +36,11 @@ struct Variant {
 };
 // Index 5 is the full-register instance of variant 0 and index 6 the same
 // with one-byte flip words; index 7 is variant 2 with the exact (6, 4, 3)
-// path for the codes that have it and 8 to
-// 11 are the column-path instances (none is chosen by kernel_variant; see
-// kernel_variant_full_regs, kernel_variant_byte_flips and
-// kernel_variant_mixed).
+// path for the codes that have it, 8 to 11 are the column-path instances (two-
+// and one-byte flip words of each) and 12 is the one for long codes (none is
+// chosen by kernel_variant; see kernel_variant_full_regs,
+// kernel_variant_byte_flips, kernel_variant_mixed, kernel_variant_columns and
+// kLongVariant).
 static const Variant kVariants[] = {{6, 4, 3}, {6, 4, 0}, {8, 4, 0}, {16, 8, 0}, {32, 16, 0}, {6, 4, 3}, {6, 4, 3},
                                     {8, 4, 0}, {6, 4, 3}, {6, 4, 3}, {10, 8, 5}, {10, 8, 5},
                                     {8, 4, 0}};

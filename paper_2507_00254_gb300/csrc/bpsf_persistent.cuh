@@ -9,8 +9,8 @@
 // iteration at a time; a work item is the initial run of a shot (with
 // oscillation counters) or one trial of a failed shot.  Per iteration a team
 // runs
-//   C phase : one thread per (slot, check): min1 / min2 / sign product over
-//             the row (Eq. c2v), one FP32 multiply by alpha, C2V messages
+//   C phase : one thread per (slot, check): V2C messages times alpha, then
+//             exclusion products under signed minima (Eq. c2v), C2V messages
 //             written in place of the V2C messages they were computed from;
 //   V phase : one thread per (slot, variable): V2C messages for the next
 //             iteration (Section II-B step 2, explicit exclusion), posterior
@@ -28,8 +28,9 @@
 // task tau = j*S + s (row j) or i*S + s (column i) addresses its data
 // directly and a warp's lanes touch consecutive words.  A lane serves one
 // slot, or 2 or 4 adjacent slots with 64- or 128-bit accesses (vector
-// phases).  Installing a slot sets its messages to the channel LLRs, so the
-// phases have no first-iteration special case.  With the layered schedule
+// phases).  Installing a slot sets its messages to the channel LLRs; where
+// these are all the same, the full-register instances' first C phase takes
+// them as an addend instead (c_row).  With the layered schedule
 // the C and V phases are replaced by layer-by-layer row updates against a
 // running posterior (vector lanes for six-wide rows, else one slot per lane).
 //
@@ -43,10 +44,13 @@
 // The manager warp does the rest of the global-memory work: it writes the
 // outboxes out, resolves the winner of each failed shot (minimum over
 // converged trials of (weight, index), merged into the shot's record by
-// atomicMin), claims new shots and trial tickets ahead of time into a small
+// atomicMin), claims new shots and trials ahead of time into a small
 // ready queue and fills the inboxes from it.  Compute warps touch global
 // memory only when a run fails (its record) or changes a decision (the
 // column's check list, in L1).
+//
+// Small launches, codes with ten ones per row and long codes run the column
+// path (bpsf_columns.cuh) in place of the team loop.
 #pragma once
 #include <cuda_runtime.h>
 
