@@ -173,6 +173,13 @@ static cudaError_t blocks_per_sm(const void *fn, int block, int smem, int *occ) 
 // One slot per team where even all trials of all shots would not fill those
 // (100 iterations of one shot 70 against 86 us), else four.  A shape with a
 // given number of blocks per SM is taken at its word.
+//
+// Exact (10, 5) codes take it at any size: on teams they have only the loop for
+// rows of up to sixteen.  [[254]] at p = 0.04, column path against the best team
+// shape: 500 shots 0.18 / 0.48 ms, 5000 0.65 / 1.55, 50 000 5.6 / 10.3; at
+// p = 0.06 50 000 shots 21.4 / 43.0.  Blocks of 24 warps instead of 19 left 72
+// registers and spilled: [[254]] 5.57 -> 5.68 ms, 3000 [[288]] shots 0.57 -> 0.64
+// (only 20 000 [[72]] shots gained, 0.94 -> 0.86).
 constexpr long long kColumnShots = 1500000;
 
 // Long codes (more than kMaxShardNnz edges; up to eight ones per row and three

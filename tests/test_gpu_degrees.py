@@ -68,6 +68,16 @@ def test_column_path(m, alpha, max_iter):
     run(rng, regular(rng, m), 4, False, alpha, max_iter)
 
 
+# The same for ten ones per row and five per column, at any batch size.
+@pytest.mark.parametrize("m,alpha,max_iter", [(16, 0.625, 40), (17, 0.0, 200), (127, 0.0, 40), (304, 0.625, 130),
+                                              (305, 0.625, 30)])
+def test_column_path_ten_ones(m, alpha, max_iter):
+    rng = np.random.default_rng(m)
+    h = regular(rng, m, 10, 5)
+    assert (h.sum(axis=0) == 5).all() and (h.sum(axis=1) == 10).all()
+    run(rng, h, 1, False, alpha, max_iter)
+
+
 # Lanes that loop over a long code's columns and rows: fewer, exactly as many and
 # more of them than lanes; column degrees 0 to 3, row degrees 2 to 8.
 @pytest.mark.parametrize("m,n,dc,alpha", [(480, 864, 8, 0.625), (432, 865, 8, 0.0), (700, 1800, 7, 0.625),
