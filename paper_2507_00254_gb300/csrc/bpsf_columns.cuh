@@ -434,7 +434,7 @@ __device__ __forceinline__ void column_loop(const StreamDev &sd, const TeamOffse
                 if (d + 1 < DV)
                     vsub<V>(pre, pre, r[d]);
                 else
-                    vsub<V>(nl, r[d], pre);  // -l_out
+                    vnegdiff<V>(nl, pre, r[d]);  // -l_out
                 if (!LONG || mp[d] >= 0) vstore<V>(reinterpret_cast<VT *>(smem + mp[d]), acc);
             }
             if (DEBUG && sd.dbg.lout) {

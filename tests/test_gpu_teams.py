@@ -1,0 +1,91 @@
+"""One prior for all columns, on teams and on the column path.  Small launches
+of exact-degree codes and long codes take the column path unless a number of
+blocks per SM is given.  Both sides round every operation alike: results,
+posteriors and flip counts equal those of the FP32 oracle, they are not close
+to it."""
+import os
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+import synth  # noqa: E402
+from oracle import Code, Params as OParams  # noqa: E402
+from paper_2507_00254_gb300 import bpsf as B  # noqa: E402
+from paper_2507_00254_gb300 import codes, harness  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+THREADS = max(1, min(16, os.cpu_count() or 1))
+
+
+class Workload:
+    """Errors at one rate for all columns, and what the oracle makes of them."""
+
+    def __init__(self, h, p, n, params, seed):
+        self.h, self.p, self.P = h, p, params
+        self.m, self.n = h.shape
+        self.code = Code(h)
+        self.s = self.code.syndrome(synth.bernoulli_bits(seed, 0, 0, n, self.n, p))
+        self.want = self.code.bpsf_batch(self.s, p, self.oparams(), fp32=True, threads=THREADS)
+        self.synd = torch.from_numpy(harness.pack_rows(self.s).view(np.int32)).cuda()
+        idx = np.concatenate([np.nonzero(r)[0] for r in h])
+        ptr = np.concatenate([[0], np.cumsum(h.sum(axis=1))])
+        self.dec = B.Decoder(ptr, idx, self.m, self.n, np.full(self.n, p), params)
+
+    def oparams(self):
+        P = self.P
+        return OParams(P.max_iter, P.alpha, P.w, P.w_max, P.short_iter, P.select, layered=P.layered)
+
+    def check(self, out, shape):
+        eo, co, io, so = self.want
+        g = {k: v.cpu().numpy() for k, v in out.items()}
+        assert (harness.unpack_rows(g["corr"].view(np.uint32), self.n) == eo).all(), shape
+        assert ((g["conv"] != 0) == co).all() and (g["iters"] == io).all() and (g["stage"] == so).all(), shape
+
+    def check_inside(self, shots):
+        """Posteriors, flip counts and Phi of some initial runs."""
+        g = {k: v.cpu().numpy() for k, v in self.dec.decode_debug(self.synd[:shots]).items()}
+        for i in range(0, shots, 7):
+            r = self.code.bp(self.s[i], self.p, self.P.max_iter, self.P.alpha, track=True, layered=self.P.layered)
+            assert (g["lout"][i] == np.asarray(r["lout"], dtype=np.float32)).all()
+            assert (g["flips"][i].astype(np.uint16) == r["flips"]).all()
+            if not r["converged"]:
+                assert (g["phi"][i] == oracle.top(r["flips"], self.P.w)).all()
+
+
+def irregular(rng, m, n, dc, dv):
+    """Row degrees 2..dc (at least one row of each end), column degrees at most dv."""
+    h = np.zeros((m, n), dtype=np.uint8)
+    for j in range(m):
+        want = dc if j == 0 else (2 if j == 1 else int(rng.integers(2, dc + 1)))
+        free = np.nonzero(h.sum(axis=0) < dv)[0]
+        h[j, rng.choice(free, size=min(want, free.size), replace=False)] = 1
+    return h
+
+
+# With one prior and alpha = 1 or 1/2 all messages are one LLR times fractions of
+# powers of two: sums cancel exactly, and zero messages of either sign meet zero
+# sums.  A zero posterior is decided 1.
+TIES = [("bb72", 0.06, 0.5), ("bb144", 0.07, 0.5), ("gb254", 0.04, 0.5), ((48, 72, 8, 4), 0.05, 1.0),
+        ((60, 80, 16, 8), 0.05, 1.0), ((432, 865, 8, 3), 0.04, 1.0)]
+
+
+@pytest.mark.parametrize("code,p,alpha", TIES, ids=str)
+def test_zero_posteriors(code, p, alpha):
+    h = codes.bb(code).dense() if isinstance(code, str) else irregular(np.random.default_rng(84), *code)
+    w = Workload(h, p, 300 if h.sum() > 2048 else 1500, B.Params(max_iter=40, alpha=alpha, w=4, short_iter=15), 7100)
+    shapes = [(1, 1, 2, 0), (1, 1, 2, 1), (1, 2, 4, 1)]
+    if h.sum(axis=1).max() == 6:
+        shapes += [(1, 4, 8, 1), (1, 8, 12, 1), (1, 8, 13, 1), (1, 2, 4, 2)]
+    for shape in shapes:
+        w.dec.tuning = shape
+        w.check(w.dec.decode(w.synd), shape)
+        w.check(w.dec.decode_debug(w.synd), shape)
+    w.dec.tuning = (1, 1, 2, 0)
+    whole = w.dec.decode(w.synd)
+    for i in range(0, 300, 3):  # three at a time: one slot per team on the column path
+        few = w.dec.decode(w.synd[i:i + 3])
+        assert all(torch.equal(few[k], whole[k][i:i + 3]) for k in few)
