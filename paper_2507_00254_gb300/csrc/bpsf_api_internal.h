@@ -106,6 +106,7 @@ inline bpsf::Records bpsf_records_carve(void *base, long long rows, int w, int W
     rec.phi = reinterpret_cast<int32_t *>(p);
     p += A(4 * r * ww);
     rec.synd = reinterpret_cast<uint32_t *>(p);
+    rec.claim = nullptr;
     rec.cap = (long long)r;
     return rec;
 }

@@ -117,11 +117,12 @@ static_assert(sizeof(StreamCounters) == 128, "counter block is two 64-byte lines
 struct Records {
     unsigned long long *qseq;   // cap: q + 1 while the record holds failure q, with kRecFree after; 0: never used
     long long *qshot;           // cap: the failed shot
-    unsigned int *done;         // cap: its trials finished (kDoneBits bits); above them, its trials claimed
+    unsigned int *done;         // cap: its trials finished (kDoneBits bits); above them, in a batch, its trials claimed
     unsigned long long *best;   // cap: min over converged trials of key << 32 | iterations
     unsigned long long *win;    // cap x Wn: min over converged trials of key << 32 | correction word
     int32_t *phi;               // cap x w
     uint32_t *synd;             // cap x Ws: the shot's syndrome
+    unsigned long long *claim;  // cap, serving only, else null: its claim word
     long long cap;              // records in the ring (a power of two)
 };
 
@@ -129,6 +130,45 @@ struct Records {
 // for each block of the launch, far below the 2^19 that the rest can count.
 constexpr int kDoneBits = 13;
 constexpr unsigned long long kRecFree = 1ull << 63;
+
+// Claims when serving.  A server's ring wraps, and a claimer that looked at a
+// record may come late: the record's trials are done, it is free, and it holds a
+// later failure or is being written.  So the trials claimed stand in one word
+// with the failure's number (record r starts with failure r's, and the last
+// trial of failure q leaves q + cap's, the next that the record can hold), and a
+// claim is a compare-and-swap on the word that was looked at: it takes trials of
+// that failure or none, and a word of another failure stays as it is.  (A
+// batch's ring never wraps: there a claim is an addition to Records::done, which
+// needs no second try.)
+constexpr int kClaimBits = 13;  // n_trials <= 4096
+
+__host__ __device__ inline unsigned long long claim_word(unsigned long long failure, int taken) {
+    return (failure << kClaimBits) | (unsigned)taken;
+}
+// Trials taken from failure q by a claim word: all T once the word is another failure's.
+__host__ __device__ inline int claim_taken(unsigned long long word, unsigned long long failure, int T) {
+    const unsigned long long low = (1ull << kClaimBits) - 1ull;
+    return (word & ~low) == claim_word(failure, 0) ? (int)(word & low) : T;
+}
+// Up to `want` of failure q's T trials: their number, the first in *first.
+// `word` is the claim word as it was seen; cas(old, next) swaps it at the record
+// and returns what it found.  A swap that fails has met another claim of the same
+// failure, so there are at most T, or the word of another, which ends the loop.
+template <typename Cas>
+__host__ __device__ inline int claim_trials(unsigned long long word, unsigned long long failure, int want, int T,
+                                            int *first, Cas cas) {
+    for (;;) {
+        const int taken = claim_taken(word, failure, T);
+        const int n = T - taken < want ? T - taken : want;
+        if (n <= 0) return 0;
+        const unsigned long long seen = cas(word, word + (unsigned)n);
+        if (seen == word) {
+            *first = taken;
+            return n;
+        }
+        word = seen;
+    }
+}
 
 constexpr int kSelKeyBits = 28;  // weight (16 bits, N <= 65535) above a 12-bit list index (n_trials <= 4096)
 

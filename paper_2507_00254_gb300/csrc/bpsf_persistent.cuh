@@ -1148,6 +1148,7 @@ __device__ __forceinline__ void shot_complete(const StreamDev &sd, long long row
 // One trial of a failed shot is over (run, or cancelled because it cannot
 // win): count it; the last one settles the winner (the minimum key of the
 // shot's converged trials) and completes the shot.
+template <bool COLS>
 __device__ __forceinline__ void trial_done(const StreamDev &sd, long long rs, long long row, long long shot,
                                            bool merged) {
     const CodeDev &cd = sd.code;
@@ -1168,9 +1169,13 @@ __device__ __forceinline__ void trial_done(const StreamDev &sd, long long rs, lo
             job.iters[row] = (int16_t)(best & 0xffffull);
             if (job.stage) job.stage[row] = 1;
         }
-        // The record is free for a later failure once its reads are done.
+        // The record is free for a later failure once its reads are done.  Its claim
+        // word is the next one's from here on (failure numbers go round the ring).
+        const unsigned long long seq = ld_vol_u64(sd.rec.qseq + rs);
+        if (!COLS && (sd.flags & kServe))
+            atomicExch(sd.rec.claim + rs, claim_word(seq - 1ull + (unsigned long long)sd.rec.cap, 0));
         __threadfence();
-        st_release_u64(sd.rec.qseq + rs, ld_vol_u64(sd.rec.qseq + rs) | kRecFree);
+        st_release_u64(sd.rec.qseq + rs, seq | kRecFree);
         shot_complete(sd, row, shot);
     }
 }
@@ -1186,7 +1191,7 @@ __device__ __forceinline__ bool trial_cannot_win(const StreamDev &sd, long long 
 // Lane-parallel write-out of outboxes that need no warp cooperation:
 // converged or uncorrectable initial runs, and trial runs.  (LONG: a converged
 // initial run's words are out already.)
-template <bool DEBUG, bool LONG>
+template <bool DEBUG, bool LONG, bool COLS>
 __device__ __forceinline__ void finalize_simple(const StreamDev &sd, TeamMem T, int s, MgrState &mg) {
     const CodeDev &cd = sd.code;
     const JobDev &job = sd.job;
@@ -1250,7 +1255,7 @@ __device__ __forceinline__ void finalize_simple(const StreamDev &sd, TeamMem T, 
         mg.trials_cancelled += 1;  // stopped: it could not win
     else
         mg.trials_local += 1;
-    trial_done(sd, rs, row, shot, conv);
+    trial_done<COLS>(sd, rs, row, shot, conv);
 }
 
 // Shots that may be claimed now.
@@ -1266,9 +1271,10 @@ __device__ __forceinline__ long long shots_available(const StreamDev &sd) {
 // may have some left.  The lanes look at the 32 records from there on, the
 // block picks among those with trials left by its number, and each record
 // picked takes one addition, which always succeeds or shows the record used
-// up.  One ticket number for all, taken by compare and swap, failed for most of
-// the blocks that raced for a failed shot's trials: 30 000 [[144]] shots at
-// p = 0.05 took 2.4 ms, and 1.85 ms with this.
+// up.  (A server's records are reused: there it is a compare-and-swap, see
+// claim_word.)  One ticket number for all, taken by compare and swap, failed for
+// most of the blocks that raced for a failed shot's trials: 30 000 [[144]] shots
+// at p = 0.05 took 2.4 ms, and 1.85 ms with this.
 //
 // While there are fewer trials than the launch has slots (128 when serving,
 // where they go before new shots), a block takes no more of them than its idle
@@ -1278,19 +1284,20 @@ __device__ __forceinline__ long long shots_available(const StreamDev &sd) {
 // at p = 0.05 took 0.37 ms with claims of up to 32 shots and take 0.34 ms;
 // four failed [[254]] shots took 525 us with claims of up to 32 trials (two
 // blocks then ran all 52) and take 102 us.
-template <bool DEBUG>
+template <bool DEBUG, bool COLS>
 __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qbase, int Q, int qstride, int lane,
                                          MgrState &mg, int n_empty, int nslots, unsigned long long head,
                                          unsigned long long rc, long long shot_next, unsigned long long wait_ns) {
     const CodeDev &cd = sd.code;
     const int Ws = cd.Ws;
+    const bool serve = !COLS && (sd.flags & kServe);  // the column path never serves
     bool got_any = false;
     int space = Q - (mg.tail - mg.head);
     unsigned long long stall = 0ull;
     if (space > 0 && cd.w > 0 && !(sd.flags & kNoTickets)) {
         const int T = cd.n_trials;
         int lim = space < 32 ? space : 32;
-        const unsigned long long few = (sd.flags & kServe) ? 128ull : (unsigned long long)gridDim.x * (unsigned)nslots;
+        const unsigned long long few = serve ? 128ull : (unsigned long long)gridDim.x * (unsigned)nslots;
         if (rc < head + 1ull + few / (unsigned)T && lim > n_empty) lim = n_empty;
         if (head < rc && lim > 0) {
             const unsigned long long q = head + (unsigned long long)lane;
@@ -1298,7 +1305,13 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
             // The record holds failure q: q + 1; it did, and all its trials are done:
             // with the kRecFree bit; it holds a later one: above; else q is not written yet.
             const unsigned long long seq = q < rc ? ld_acquire_u64(sd.rec.qseq + rs) : 0ull;
-            const bool left = seq == q + 1ull && (int)(ld_vol_u32(sd.rec.done + rs) >> kDoneBits) < T;
+            unsigned long long word = 0ull;
+            int taken = T;
+            if (seq == q + 1ull) {
+                if (serve) word = ld_vol_u64(sd.rec.claim + rs);
+                taken = serve ? claim_taken(word, q, T) : (int)(ld_vol_u32(sd.rec.done + rs) >> kDoneBits);
+            }
+            const bool left = taken < T;
             const bool unwritten = (seq & ~kRecFree) < q + 1ull;
             const unsigned lm = __ballot_sync(FULLMASK, left);
             // Records used up from the head on.
@@ -1311,7 +1324,11 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
                 int nth = rank - (int)(blockIdx.x % (unsigned)n);  // the lane's place in the block's order
                 if (nth < 0) nth += n;
                 const int want = lim - nth * T < T ? lim - nth * T : T;
-                if (left && want > 0) {
+                if (left && want > 0 && serve) {
+                    got = claim_trials(word, q, want, T, &k0, [&](unsigned long long old, unsigned long long next) {
+                        return atomicCAS(sd.rec.claim + rs, old, next);
+                    });
+                } else if (left && want > 0) {
                     k0 = (int)(atomicAdd(&sd.rec.done[rs], (unsigned)want << kDoneBits) >> kDoneBits);
                     got = T - k0 < want ? (T - k0 > 0 ? T - k0 : 0) : want;
                 }
@@ -1337,6 +1354,7 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
                     mine_rs = r;
                 }
             }
+            __syncwarp();  // the claiming lane's acquire of the record holds for the lanes that read it
             if (lane < take) {
                 rs = mine_rs;
                 QEntry *e = qentry(qbase, (mg.tail + lane) % Q, qstride);
@@ -1371,7 +1389,7 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
                         for (int w = 0; w < Ws; ++w) sd.dbg.trial_synd[(shot * T + kidx) * Ws + w] = sy[w];
                 } else {
                     // Early cancel: counted as done, not run.
-                    trial_done(sd, rs, row_of(sd, shot), shot, false);
+                    trial_done<COLS>(sd, rs, row_of(sd, shot), shot, false);
                     ++mg.trials_cancelled;
                     e->kind = 0;
                 }
@@ -1397,7 +1415,7 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
         }
     }
     mg.stall_q = stall;
-    if (space > 0 && ((sd.flags & kServe) || shot_next < sd.job.n_shots)) {
+    if (space > 0 && (serve || shot_next < sd.job.n_shots)) {
         long long c0 = 0;
         int got = 0;
         if (lane == 0) {
@@ -1412,7 +1430,7 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
                     want = want < n_empty ? want : n_empty;
                     if (want == 0) break;
                 }
-                if (sd.flags & kServe) {
+                if (serve) {
                     // More shots may be published later: claim none that are not yet.
                     if (want > left) want = left;
                     const long long seen = (long long)atomicCAS(&sd.ctr->shot_next, (unsigned long long)cur,
@@ -1467,7 +1485,7 @@ __device__ __forceinline__ bool prefetch(const StreamDev &sd, unsigned char *qba
     return got_any;
 }
 
-template <bool DEBUG, bool LONG>
+template <bool DEBUG, bool LONG, bool COLS>
 __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned char *team_base, int team_bytes,
                              const TeamOffsets &to, int teams, int S, unsigned char *qbase, int Q, BlockHdr *hdr,
                              int lane, unsigned long long wait_ns) {
@@ -1501,7 +1519,7 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
                 if (T.st[s].cancel != key && trial_cannot_win(sd, T.st[s].rec, kidx))
                     *reinterpret_cast<volatile long long *>(&T.st[s].cancel) = key;
             }
-            if (fin) finalize_simple<DEBUG, LONG>(sd, T, s, mg);
+            if (fin) finalize_simple<DEBUG, LONG, COLS>(sd, T, s, mg);
             __syncwarp();
             if (fin) {
                 __threadfence_block();
@@ -1543,7 +1561,7 @@ __device__ void manager_loop(const StreamDev &sd, const LayoutMem &L, unsigned c
         }
         __syncwarp();
         // (C) claim work ahead.
-        if (prefetch<DEBUG>(sd, qbase, Q, qstride, lane, mg, n_empty, nslots, rec_head, rec_count, shot_next, wait_ns))
+        if (prefetch<DEBUG, COLS>(sd, qbase, Q, qstride, lane, mg, n_empty, nslots, rec_head, rec_count, shot_next, wait_ns))
             progress = true;
         // Count finished initial runs once no new shot can be claimed.
         if (!serve && shot_next >= sd.job.n_shots) {
@@ -1804,7 +1822,7 @@ __global__ void __launch_bounds__(COLS ? (DVX > 0 ? kColumnThreads : kLongThread
         L.lch = reinterpret_cast<const float *>(lay + lo.lch);
         L.lch_pos = reinterpret_cast<const float *>(lay + lo.lch_pos);
         if (warp == 0) {
-            manager_loop<DEBUG, kPath == kPathLong>(sd, L, team_base, to.total, to, teams, S, qbase, Q, hdr, lane, kp.wait_ns);
+            manager_loop<DEBUG, kPath == kPathLong, COLS>(sd, L, team_base, to.total, to, teams, S, qbase, Q, hdr, lane, kp.wait_ns);
         } else {
             const int team = (warp - 1) / W;
             if (team < teams) {

@@ -238,13 +238,17 @@ extern "C" bpsf_status bpsf_serve_start(bpsf_server **out, bpsf_ctx *const *code
         if (e != cudaSuccess) break;
         // A ring of failed-shot records (failed shots in flight never
         // outnumber admitted shots), all free.
-        // A claim reads a record's number and its count one after the other: with
-        // at least 1024 records none is reused in between.
-        const long long RR = bpsf_record_ring(std::max<long long>((long long)R, 1024));
-        e = cudaMalloc(&sc.d_rec, bpsf_records_bytes(RR, x->p.w, x->Ws, x->Wn, 16));
+        const long long RR = bpsf_record_ring((long long)R);
+        const size_t rec_bytes = a16(bpsf_records_bytes(RR, x->p.w, x->Ws, x->Wn, 16));
+        e = cudaMalloc(&sc.d_rec, rec_bytes + 8 * (size_t)RR);
         if (e != cudaSuccess) break;
         sc.rec = bpsf_records_carve(sc.d_rec, RR, x->p.w, x->Ws, x->Wn, 16);
+        sc.rec.claim = reinterpret_cast<unsigned long long *>(static_cast<unsigned char *>(sc.d_rec) + rec_bytes);
         e = cudaMemset(sc.rec.qseq, 0, 8 * (size_t)RR);
+        std::vector<unsigned long long> claims((size_t)RR);
+        for (long long r = 0; r < RR; ++r) claims[r] = claim_word((unsigned long long)r, 0);
+        if (e == cudaSuccess) e = cudaMemcpy(sc.rec.claim, claims.data(), 8 * (size_t)RR, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) break;
         // The serving stream of this code.
         JobDev job{sc.m_synd, sc.m_corr, sc.m_conv, sc.m_iters, sc.m_stage8, 0, x->Ws, x->Wn};
         StreamDev sd = bpsf_make_stream(x, job, nullptr, kServe);

@@ -236,3 +236,31 @@ def test_replays_time_both_forms_on_one_clock(mix):
     assert span_s >= arrivals[-1]
     with pytest.raises(B.BpsfError):
         B.plain_replay(decs, arrivals[::-1].copy(), which, reqs)  # arrivals must not decrease
+
+
+def test_record_ring_wraps_over_many_failures(mix):
+    """Sixteen rows, so sixteen failed-shot records, taken by hundreds of failures
+    in turn: every claim takes trials of the failure it looked at."""
+    decs = [d for _, _, d, _ in mix]
+    srv = B.Server(decs, max_inflight_shots=16)
+    try:
+        synds = [synd_host(c, d, q, n, 7900 + k)
+                 for k, ((_, c, d, _), q, n) in enumerate(zip(mix, (0.1, 0.1, 0.012), (800, 600, 200)))]
+        refs = [alone(d, s) for d, s in zip(decs, synds)]
+        for r, least in zip(refs, (400, 300, 0)):
+            assert (r["stage"] != 0).sum() > least  # failed initial runs (few of the third code)
+        window, got, at, step = [], [[], [], []], [0, 0, 0], 0
+        while window or any(a < s.shape[0] for a, s in zip(at, synds)):
+            for k, s in enumerate(synds):
+                n = min(1 + (step + k) % 4, s.shape[0] - at[k])
+                if n > 0 and sum(w[0] == k for w in window) < 4:
+                    window.append((k, n, srv.submit(k, s[at[k]:at[k] + n])))
+                    at[k] += n
+            step += 1
+            if step % 3 == 0 or len(window) > 9 or all(a == s.shape[0] for a, s in zip(at, synds)):
+                k, n, t = window.pop(0)
+                got[k].append(srv.poll(t, n, k))
+        for k, ref in enumerate(refs):
+            same({key: np.concatenate([g[key] for g in got[k]]) for key in ref}, ref)
+    finally:
+        srv.stop()
