@@ -89,3 +89,90 @@ def test_zero_posteriors(code, p, alpha):
     for i in range(0, 300, 3):  # three at a time: one slot per team on the column path
         few = w.dec.decode(w.synd[i:i + 3])
         assert all(torch.equal(few[k], whole[k][i:i + 3]) for k in few)
+
+
+_cache = {}
+
+
+def workload(name, alpha, max_iter=100):
+    """Two thousand shots of a code whose runs often fail; kept for the module."""
+    key = (name, alpha, max_iter)
+    if key not in _cache:
+        p = {"bb72": 0.06, "bb144": 0.07, "gb254": 0.04}[name]
+        P = B.Params(max_iter=max_iter, alpha=alpha, w=5, short_iter=20)
+        w = Workload(codes.bb(name).dense(), p, 2000, P, 7100)
+        assert (w.want[3] != 0).sum() > 10  # failed initial runs among them
+        _cache[key] = w
+    return _cache[key]
+
+
+# (W, S, B, blocks per SM, iteration chunk).  One block per SM takes the
+# full-register instance, two or more the 64-register one; thirteen teams of
+# eight slots fit with one-byte flip words only.
+TEAMS = [(1, 1, 4, 1), (1, 2, 15, 1), (1, 4, 15, 1), (1, 8, 12, 1), (1, 8, 13, 1), (1, 8, 13, 1, 2), (1, 16, 4, 1),
+         (1, 32, 2, 1), (2, 2, 8, 1), (2, 8, 8, 1, 2), (4, 1, 12, 1, 3), (4, 16, 12, 1), (8, 1, 8, 1), (8, 32, 8, 1),
+         (1, 32, 3, 1, 64), (1, 4, 15, 1, 8), (1, 4, 4, 2), (2, 2, 8, 2), (1, 1, 8, 2)]
+
+
+@pytest.mark.parametrize("alpha", [0.625, 0.0])
+@pytest.mark.parametrize("shape", TEAMS, ids=str)
+def test_six_ones_per_row(shape, alpha):
+    w = workload("bb144", alpha)
+    w.dec.tuning = shape
+    w.check(w.dec.decode(w.synd), shape)
+
+
+@pytest.mark.parametrize("alpha", [0.625, 0.0])
+@pytest.mark.parametrize("shape", [(1, 1, 4, 1), (1, 4, 12, 1), (1, 8, 12, 1), (1, 8, 13, 1), (2, 2, 8, 2)], ids=str)
+def test_inside_six_ones_per_row(shape, alpha):
+    w = workload("bb144", alpha)
+    w.dec.tuning = shape
+    w.check_inside(350)
+
+
+def test_two_byte_flip_words():
+    """More than 127 iterations: the shape for one-byte words is refused, the others count in two bytes."""
+    w = workload("bb144", 0.625, 200)
+    with pytest.raises(B.BpsfError):
+        w.dec.tuning = (1, 8, 13, 1)
+    for shape in ((1, 8, 12, 1), (1, 2, 4, 2)):
+        w.dec.tuning = shape
+        w.check(w.dec.decode(w.synd), shape)
+        w.check_inside(100)
+
+
+@pytest.mark.parametrize("alpha", [0.625, 0.0])
+@pytest.mark.parametrize("shape", [(1, 1, 8, 1), (1, 2, 8, 1), (1, 4, 8, 1), (1, 8, 4, 1), (2, 16, 2, 1), (4, 2, 8, 2)],
+                         ids=str)
+def test_ten_ones_per_row(shape, alpha):
+    w = workload("gb254", alpha)
+    w.dec.tuning = shape
+    w.check(w.dec.decode(w.synd), shape)
+    w.check_inside(70)
+
+
+# Row degrees 2 to dc, column degrees at most dv, one prior for all columns: the
+# first iteration has no message set-up on teams, and one magnitude on the long
+# codes' loop (the last two, where no blocks per SM are given).
+@pytest.mark.parametrize("m,n,dc,dv", [(37, 60, 6, 3), (37, 60, 8, 4), (37, 80, 16, 8), (37, 90, 20, 16),
+                                       (480, 864, 8, 3), (432, 865, 8, 3)])
+@pytest.mark.parametrize("alpha", [0.625, 0.0])
+def test_one_prior(m, n, dc, dv, alpha):
+    h = irregular(np.random.default_rng(1000 * dc + n), m, n, dc, dv)
+    w = Workload(h, 0.04, 300, B.Params(max_iter=40, alpha=alpha, w=3, short_iter=9), 7200 + n)
+    for shape in ((1, 1, 2, 1), (1, 2, 4, 1), (2, 4, 4, 1), (2, 2, 4, 0)):
+        if m > 100 and shape[1] > 2:
+            continue  # no room for four slots of a long code in two teams
+        w.dec.tuning = shape
+        w.check(w.dec.decode(w.synd), shape)
+        w.check_inside(70)
+
+
+def test_uneven_codes_in_one_launch():
+    """Exact codes beside the phenomenological one: the instance with both team loops."""
+    P = B.Params(max_iter=100, alpha=0.0, w=5, short_iter=20)
+    works = [workload("bb72", 0.0), Workload(codes.phenom("bb144").dense(), 0.004, 1200, P, 7300), workload("bb144", 0.0)]
+    for w, shape in zip(works, ((1, 2, 4, 1), (2, 1, 4, 1), (1, 4, 4, 1))):
+        w.dec.tuning = shape
+    for w, out in zip(works, B.decode_multi([w.dec for w in works], [w.synd for w in works])):
+        w.check(out, "mixed")
