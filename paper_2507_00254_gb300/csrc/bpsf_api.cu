@@ -1063,9 +1063,10 @@ extern "C" bpsf_status bpsf_decode_plain(bpsf_ctx *c, int64_t n, const uint32_t 
     if (st != BPSF_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
     bpsf_ctx *cs1[1] = {c};
-    // Launch A: one block, one team, one slot, the initial run of one shot.
+    // Launch A: one block, one team, one slot, the initial run of one shot.  It keeps
+    // the shape's blocks per SM: where these are given, both launches are teams.
     bpsf_plan plA, plB;
-    bpsf_tuning tA{c->tune.warps_per_team, 1, c->tune.warps_per_team, 0, 1};
+    bpsf_tuning tA{c->tune.warps_per_team, 1, c->tune.warps_per_team, c->tune.blocks_per_sm, 1};
     const long long one_shot[1] = {1};
     st = bpsf_make_plan(cs1, 1, &tA, false, &plA, false, one_shot);
     if (st != BPSF_OK) return st;

@@ -176,3 +176,19 @@ def test_uneven_codes_in_one_launch():
         w.dec.tuning = shape
     for w, out in zip(works, B.decode_multi([w.dec for w in works], [w.synd for w in works])):
         w.check(out, "mixed")
+
+
+def test_plain_form_takes_the_given_shape():
+    """Blocks per SM given: the initial runs of the plain form are teams of one slot.  (With
+    4095 trials the column path would hold four slots, three of them idle.)"""
+    P = B.Params(max_iter=60, alpha=0.625, w=12, short_iter=3)
+    w = Workload(codes.bb("bb144").dense(), 0.02, 40, P, 7400)
+    conv = np.nonzero(w.want[3] == 0)[0]
+    assert conv.size > 20
+    for shape in ((1, 4, 8, 1), (2, 2, 4, 2)):
+        w.dec.tuning = shape
+        out = w.dec.decode(w.synd[torch.from_numpy(conv).cuda()].contiguous(), plain=True, sync=False)
+        assert (out["iters"].cpu().numpy() == w.want[2][conv]).all() and (out["stage"] == 0).all()
+        work = w.dec.last_work()
+        assert work["iterations"] == w.want[2][conv].sum() and work["slot_capacity"] == work["iterations"]
+        w.check(w.dec.decode(w.synd, plain=True), shape)
