@@ -217,7 +217,8 @@ static bool plan_long(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tu
 }
 
 static void plan_columns(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, const long long *shots,
-                         int dc, int dv, bpsf_plan *out, int *variant, int *B, int *smem, long long *grid_max, int Q) {
+                         bool trials, int dc, int dv, bpsf_plan *out, int *variant, int *B, int *smem,
+                         long long *grid_max, int Q) {
     if (kernel_variant_columns(dc, dv, 2) < 0) return;
     long long work = 0;
     int fb = 1;
@@ -233,7 +234,7 @@ static void plan_columns(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning 
     for (int k = 0; k < n_codes; ++k) {
         const bpsf_ctx *c = codes[k];
         const int W = (c->N + 31) / 32, teams = std::min(kMaxNamedTeams, kMaxColumnWarps / W);
-        const long long runs = std::min(shots[k], kColumnShots) * (1 + c->n_trials);
+        const long long runs = std::min(shots[k], kColumnShots) * (1 + (trials ? c->n_trials : 0));
         const int S = runs <= (long long)teams * c->sm_count ? 1 : 4;
         out->W_code[k] = W;
         out->S_code[k] = S;
@@ -250,7 +251,7 @@ static void plan_columns(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning 
 }
 
 bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, bool debug,
-                           bpsf_plan *out, bool shrink, const long long *shots) {
+                           bpsf_plan *out, bool shrink, const long long *shots, bool trials) {
     // One kernel variant must fit every code of the launch.
     bool all_regular = true, layered = false;
     int dc = 0, dv = 0, B = 0, bps = 0;
@@ -328,7 +329,7 @@ bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tunin
     long long grid_max = 1ll << 30;
     if (shots && plan_long(codes, n_codes, tunes, shots, all_regular && dc == 6 && dv == 3, out, &variant, &B, &smem, Q)) {
     } else if (shots && all_regular && !layered)
-        plan_columns(codes, n_codes, tunes, shots, dc, dv, out, &variant, &B, &smem, &grid_max, Q);
+        plan_columns(codes, n_codes, tunes, shots, trials, dc, dv, out, &variant, &B, &smem, &grid_max, Q);
     bpsf_status st = bpsf_ensure_kernel_attrs(variant, c0->smem_optin);
     if (st != BPSF_OK) return st;
     const int block = 32 * (B + 1);
@@ -1068,7 +1069,7 @@ extern "C" bpsf_status bpsf_decode_plain(bpsf_ctx *c, int64_t n, const uint32_t 
     bpsf_plan plA, plB;
     bpsf_tuning tA{c->tune.warps_per_team, 1, c->tune.warps_per_team, c->tune.blocks_per_sm, 1};
     const long long one_shot[1] = {1};
-    st = bpsf_make_plan(cs1, 1, &tA, false, &plA, false, one_shot);
+    st = bpsf_make_plan(cs1, 1, &tA, false, &plA, false, one_shot, false);
     if (st != BPSF_OK) return st;
     // Launch B: the shot's trials spread over blocks of the tuned shape.
     st = bpsf_make_plan(cs1, 1, &c->tune, false, &plB, false, one_shot);

@@ -140,9 +140,11 @@ bpsf_status bpsf_ensure_kernel_attrs(int variant, int smem_optin);
 // Plan one launch over n_codes codes; tunes[k] is code k's team shape (a
 // single tuning for a one-code launch).  With shrink, a code whose block does
 // not fit gets fewer slots per team, then fewer teams.  shots: the shots of
-// each code in a batch launch (the column path serves small ones), or null.
+// each code in a batch launch (the column path serves small ones), or null;
+// trials: the launch also runs the trials of failed shots.
 bpsf_status bpsf_make_plan(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, bool debug,
-                           bpsf_plan *out, bool shrink = false, const long long *shots = nullptr);
+                           bpsf_plan *out, bool shrink = false, const long long *shots = nullptr,
+                           bool trials = true);
 void bpsf_launch_plan(const bpsf_plan &pl, bool debug, bpsf::StreamDev *sds, int n, int grid, void *stream);
 bool bpsf_tuning_cache_lookup(const bpsf_ctx *c, bpsf_tuning *out);
 bpsf::StreamDev bpsf_make_stream(const bpsf_ctx *c, const bpsf::JobDev &job, const bpsf::DebugDev *dbg,

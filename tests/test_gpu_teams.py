@@ -192,3 +192,13 @@ def test_plain_form_takes_the_given_shape():
         work = w.dec.last_work()
         assert work["iterations"] == w.want[2][conv].sum() and work["slot_capacity"] == work["iterations"]
         w.check(w.dec.decode(w.synd, plain=True), shape)
+
+
+def test_plain_form_runs_one_shot_on_one_slot():
+    """However many trials a code has, an initial run of the plain form leaves no slot idle."""
+    P = B.Params(max_iter=60, alpha=0.625, w=12, short_iter=3)
+    w = Workload(codes.bb("bb144").dense(), 0.02, 40, P, 7400)
+    synd = w.synd[torch.from_numpy(np.nonzero(w.want[3] == 0)[0]).cuda()].contiguous()
+    w.dec.decode(synd, plain=True, sync=False)
+    work = w.dec.last_work()
+    assert work["iterations"] > 0 and work["slot_capacity"] == work["iterations"]
