@@ -4,6 +4,7 @@ input before any device work."""
 import ctypes as C
 import os
 import re
+import types
 
 import numpy as np
 import pytest
@@ -142,3 +143,17 @@ def test_multi_job_calls_reject_bad_job_lists():
         assert fn(1, one, None) == B.BPSF_EINVAL  # NULL context
         many = (B.bpsf_job * 17)()
         assert fn(17, many, None) == B.BPSF_EINVAL  # more than 16 jobs
+
+
+@pytest.mark.parametrize("n", [0, 1, 7, 4096, 4097])
+def test_outputs_are_tensors_of_their_own(n):
+    """Zeros, each in a storage of its own size: saving or resizing one leaves the others alone."""
+    torch = pytest.importorskip("torch")
+    out = B.Decoder.outputs(types.SimpleNamespace(Wn=5), n, "cpu")
+    want = dict(corr=((n, 5), torch.int32), conv=((n,), torch.uint8), iters=((n,), torch.int16),
+                stage=((n,), torch.uint8))
+    assert list(out) == list(want)
+    for key, t in out.items():
+        assert (tuple(t.shape), t.dtype) == want[key] and t.is_contiguous() and not t.any()
+        assert t.storage_offset() == 0 and t.untyped_storage().nbytes() == t.numel() * t.element_size()
+    assert n == 0 or len({t.data_ptr() for t in out.values()}) == 4
