@@ -254,13 +254,16 @@ bpsf_status bpsf_sync(bpsf_ctx *ctx, void *stream);
  * layered schedule, a kernel instance with one-byte flip counters makes
  * room for shapes that two-byte counters do not fit (for example 13 teams of
  * 8 slots on [[144,12,12]]).
- * Small batches (up to about 1.5 * 10^6 shots times columns in a launch, for
- * example 10^4 shots of [[144,12,12]]) of codes of row weight 6 and column
- * weight 3 without the layered schedule run with a lane per column instead, on
- * a shape of their own, unless blocks_per_sm is given.  So do batches of any
- * size of codes with ten ones in every row and five in every column, and of
- * long codes (more than 2048 ones in H, at most eight in a row and three in a
- * column, not all rows with six and columns with three).  Results do not depend on it.
+ * Small batches (up to 1.5 * 10^6 shots times columns in a launch, for example
+ * 10^4 shots of [[144,12,12]]) of codes of row weight 6 and column weight 3
+ * without the layered schedule run with a lane per column instead, on a shape of
+ * their own, unless blocks_per_sm is given: of codes of up to 608 columns, and of
+ * longer ones with more than 2048 ones in H.  So do batches of any size of codes
+ * of up to 608 columns with ten ones in every row and five in every column, and
+ * of long codes (more than 2048 ones in H, at most eight in a row and three in a
+ * column) whose four slots fit in the shared memory of a block (about 172 KB for
+ * 864 x 2592 with 6840 ones).  The server always runs on teams.  Results do not
+ * depend on it.
  */
 typedef struct {
     int32_t warps_per_team;  /* 1, 2, 4 or 8 */
@@ -278,13 +281,19 @@ bpsf_status bpsf_get_tuning(const bpsf_ctx *ctx, bpsf_tuning *out);
 bpsf_status bpsf_set_tuning(bpsf_ctx *ctx, const bpsf_tuning *t);
 
 /*
- * Autotuner: times bpsf_decode over candidate launch shapes on n_sample
+ * Autotuner: times decodes on teams over candidate launch shapes on n_sample
  * syndromes of random errors drawn at rate p_sample (device generator):
  * threads per shot (warps per team over slots per team), shots per block
  * (slots per team x teams), then the iteration chunk for the fastest shape.
  * Keeps the fastest, sets it on ctx and caches it per code shape (M, N, nnz,
  * degrees, parameters) for the process; a context created later for the same
  * code shape starts with it.  Synchronises `stream`.  chosen is nullable.
+ * A shape with blocks_per_sm = 0 governs the launches that run on teams (see
+ * bpsf_tuning): for row weight 6 and column weight 3 the batches above the
+ * small ones, whatever n_sample is.  Codes that have a shape of their own at
+ * every batch size keep it (the tuning then stays as it was, with
+ * blocks_per_sm = 0), unless a team shape is at least 3 % faster on the sample:
+ * that one is set with its blocks per SM, so that it is taken.
  */
 bpsf_status bpsf_autotune(bpsf_ctx *ctx, double p_sample, int64_t n_sample, void *stream, bpsf_tuning *chosen);
 

@@ -1380,7 +1380,6 @@ extern "C" bpsf_status bpsf_autotune(bpsf_ctx *c, double p_sample, int64_t n_sam
     float best_ms = 1e30f;
     bpsf_status st = BPSF_OK;
     bpsf_ctx *cs1[1] = {c};
-    c->team_only = true;  // the shapes apply to the team path
     // Time one shape: the best of two decodes after a warm-up decode.
     auto time_shape = [&](const bpsf_tuning &t) -> float {
         c->tune = t;
@@ -1396,6 +1395,21 @@ extern "C" bpsf_status bpsf_autotune(bpsf_ctx *c, double p_sample, int64_t n_sam
         }
         return ms_min;
     };
+    // A code whose launches of any size have a shape of their own keeps it, unless a
+    // team shape is faster by more than the timing's noise.
+    bpsf_tuning own = saved;
+    own.blocks_per_sm = 0;
+    bool has_own = false;
+    {
+        const long long any[1] = {1ll << 40};
+        bpsf_plan pl;
+        has_own = bpsf_make_plan(cs1, 1, &own, false, &pl, false, any) == BPSF_OK && kernel_variant_own_shape(pl.variant);
+    }
+    if (has_own) {
+        best = own;
+        best_ms = 0.97f * time_shape(own);
+    }
+    c->team_only = true;  // the other candidates are team shapes
     // Threads per shot and shots per block: warps per team, slots per team and
     // compute warps per block, every shape that fits.
     const int Ws_[] = {1, 2, 4, 8};
@@ -1413,11 +1427,12 @@ extern "C" bpsf_status bpsf_autotune(bpsf_ctx *c, double p_sample, int64_t n_sam
                 if (st == BPSF_OK && ms < best_ms) {
                     best_ms = ms;
                     best = t;
+                    if (has_own) best.blocks_per_sm = std::max(1, pl.grid / c->sm_count);  // else not taken
                 }
             }
     // The iteration chunk of the fastest shape.
     for (int k : {2, 4, 8}) {
-        if (st != BPSF_OK || best_ms >= 1e30f) break;
+        if (st != BPSF_OK || best_ms >= 1e30f || (has_own && best.blocks_per_sm == 0)) break;
         bpsf_tuning t = best;
         t.iter_chunk = k;
         const float ms = time_shape(t);

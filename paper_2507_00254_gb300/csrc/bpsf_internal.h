@@ -397,6 +397,7 @@ int kernel_variant_dv(int variant);          // column table width of a variant
 int kernel_variant_full_regs(int variant);   // its one-block, full-register instance
 int kernel_variant_byte_flips(int variant);  // its one-block instance with one-byte flip words, -1 if none
 int kernel_variant_columns(int dc, int dv, int fb);  // column-path instance of an exact code, -1 if none
+bool kernel_variant_own_shape(int variant);   // an instance whose launches have a shape of their own (columns, long codes)
 int kernel_variant_mixed(int variant);       // its instance with the exact (6, 4, 3) path as well, -1 if none
 const void *persistent_kernel_ptr(int variant, bool debug, bool layered);
 void launch_persistent(int variant, bool debug, bool layered, int grid, int block, int smem, const LaunchArgs &args,

@@ -97,6 +97,8 @@ int kernel_variant_columns(int dc, int dv, int fb) {
     return -1;
 }
 
+bool kernel_variant_own_shape(int variant) { return variant >= 8; }
+
 // The instance that runs variant 2's codes together with exact (6, 4, 3)
 // codes on their own path, or -1.
 int kernel_variant_mixed(int variant) { return variant == 2 ? 7 : -1; }

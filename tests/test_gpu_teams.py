@@ -202,3 +202,16 @@ def test_plain_form_runs_one_shot_on_one_slot():
     w.dec.decode(synd, plain=True, sync=False)
     work = w.dec.last_work()
     assert work["iterations"] > 0 and work["slot_capacity"] == work["iterations"]
+
+
+@pytest.mark.parametrize("code,p,shots", [("gb254", 0.04, 4000), ((432, 865, 8, 3), 0.02, 1000)], ids=str)
+def test_autotuned_shape_is_the_one_that_decodes(code, p, shots):
+    """Codes with a shape of their own at any batch size: the autotuner leaves it, or sets a
+    faster team shape with its blocks per SM."""
+    h = codes.bb(code).dense() if isinstance(code, str) else irregular(np.random.default_rng(84), *code)
+    w = Workload(h, p, 300, B.Params(max_iter=30, alpha=0.625, w=2, short_iter=9), 7500)
+    before = w.dec.tuning
+    chosen = w.dec.autotune(p_sample=p, n_sample=shots)
+    assert w.dec.tuning == chosen and (chosen == before or chosen[3] > 0)
+    assert before[3] == 0
+    w.check(w.dec.decode(w.synd), chosen)
