@@ -6,7 +6,8 @@ decoded with normalised min-sum (alpha 0.625, max_iter 100), |Phi| = 6
 (63 trials per failed shot, short_iter 20), minimum-weight selection.  All
 four batches and all trials run in ONE persistent launch per step.
 
-Prints one JSON line.  ``--impl reference`` times the CPU oracle instead (the
+Prints the headline as one JSON line on stdout (secondary measurements as one on
+stderr).  ``--impl reference`` times the CPU oracle instead (the
 reference arm: a plain C implementation run on the host cores).
 """
 from __future__ import annotations
@@ -203,6 +204,19 @@ def oracle_plan():
         e = synth.bernoulli_bits(synth.SEEDS["mixed"][k], 0, 0, 4000, oc.N, 0.05)
         out["config4_%s_p0.05" % name] = case(oc, oc.syndrome(e), 0.05, op(PARAMS), 300, 4000)
     return out
+
+
+# The keys of the one line on stdout; a reader that keeps only the end of the
+# output still gets all of it (the whole of the measurements is some 22 KB).
+HEADLINE = ("impl", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "roofline", "cpu_baseline", "e2e", "gpu_launches", "clocks",
+            "latency_ms", "ler")
+
+
+def emit(results):
+    """The headline as one JSON line on stdout; everything else as one JSON line on stderr before it."""
+    print(json.dumps({"secondary": {k: v for k, v in results.items() if k not in HEADLINE}}), file=sys.stderr, flush=True)
+    print(json.dumps({k: results[k] for k in HEADLINE if k in results}), flush=True)
 
 
 def run_reference(args, rank, world):
@@ -426,9 +440,7 @@ def run_gpu(args, rank, world, pool):
             "roofline": {"bound": "smem", "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gedge-updates/s",
                          "frac": achieved / peak, "traffic": traffic, "traffic_unit": "bytes per launch",
                          "note": ("peak = SMs x 128 B/clk shared memory / 16 B per edge-update at the max SM clock "
-                                  "(nominal shared-memory bandwidth, no measured figure exists for it); the ncu "
-                                  "counters read the kernel as latency-bound (issue and shared-memory wavefronts "
-                                  "both near half of peak), not bandwidth-bound")},
+                                  "(nominal, no measured figure exists for it)")},
             "cpu_baseline": cpu,
             "e2e": {"value": shots_step / e2e_dt, "unit": "shots/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h},
@@ -447,7 +459,7 @@ def run_gpu(args, rank, world, pool):
             "input_gen_s": t_gen, "wall_timed_s": t_wall,
         }
         line.update(extras)
-        print(json.dumps(line), flush=True)
+        emit(line)
     if dist:
         dist.barrier()
         dist.destroy_process_group()
@@ -455,7 +467,7 @@ def run_gpu(args, rank, world, pool):
 
 
 # --------------------------------------------------------------------------
-# Secondary measurements (reported beside the headline line)
+# Secondary measurements (the JSON line on stderr)
 # --------------------------------------------------------------------------
 
 SERVE_BB = ("bb72", "bb90", "bb108", "bb144", "bb288")

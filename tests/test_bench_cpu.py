@@ -40,3 +40,17 @@ def test_reference_arm_prints_one_contract_line():
     assert d["cpu_baseline"]["value"] == d["value"]
     assert d["e2e"] == {"value": d["value"], "unit": "shots/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}
     assert d["config"]["sample_shots_per_p"] == 100
+
+
+def test_headline_is_one_short_line(capsys):
+    """The contract's keys on stdout, the rest on stderr: the whole together is more than a log's tail keeps."""
+    contract = ["metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "config", "roofline", "cpu_baseline", "e2e", "gpu_launches", "clocks"]
+    results = {k: "x" * 60 for k in contract}
+    results.update(latency_ms={"batched_step_p50": 1.0}, served={"rows": ["y" * 100] * 90}, work={"iterations": 3})
+    bench.emit(results)
+    out, err = capsys.readouterr()
+    assert len(out.splitlines()) == 1 and len(out) < 2500
+    line = json.loads(out)
+    assert all(line[k] == results[k] for k in contract) and "served" not in line
+    assert json.loads(err)["secondary"] == {"served": results["served"], "work": results["work"]}
