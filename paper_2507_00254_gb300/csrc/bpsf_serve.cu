@@ -245,9 +245,13 @@ extern "C" bpsf_status bpsf_serve_start(bpsf_server **out, bpsf_ctx *const *code
         sc.rec = bpsf_records_carve(sc.d_rec, RR, x->p.w, x->Ws, x->Wn, 16);
         sc.rec.claim = reinterpret_cast<unsigned long long *>(static_cast<unsigned char *>(sc.d_rec) + rec_bytes);
         e = cudaMemset(sc.rec.qseq, 0, 8 * (size_t)RR);
-        std::vector<unsigned long long> claims((size_t)RR);
-        for (long long r = 0; r < RR; ++r) claims[r] = claim_word((unsigned long long)r, 0);
-        if (e == cudaSuccess) e = cudaMemcpy(sc.rec.claim, claims.data(), 8 * (size_t)RR, cudaMemcpyHostToDevice);
+        // Record r starts with failure r's claim word (a piece at a time: the ring may be large).
+        unsigned long long piece[2048];
+        for (long long r = 0; r < RR && e == cudaSuccess; r += 2048) {
+            const long long m = std::min<long long>(2048, RR - r);
+            for (long long k = 0; k < m; ++k) piece[k] = claim_word((unsigned long long)(r + k), 0);
+            e = cudaMemcpy(sc.rec.claim + r, piece, 8 * (size_t)m, cudaMemcpyHostToDevice);
+        }
         if (e != cudaSuccess) break;
         // The serving stream of this code.
         JobDev job{sc.m_synd, sc.m_corr, sc.m_conv, sc.m_iters, sc.m_stage8, 0, x->Ws, x->Wn};
@@ -261,6 +265,8 @@ extern "C" bpsf_status bpsf_serve_start(bpsf_server **out, bpsf_ctx *const *code
         sd.serve.idle_ns = s->idle_ns;
         s->sds[k] = sd;
     }
+    // The loop runs on a stream that does not wait for the resets above.
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
         free_server(s);
         return bpsf_fail(BPSF_ENOMEM, "serving buffers: %s", cudaGetErrorString(e));

@@ -264,3 +264,18 @@ def test_record_ring_wraps_over_many_failures(mix):
             same({key: np.concatenate([g[key] for g in got[k]]) for key in ref}, ref)
     finally:
         srv.stop()
+
+
+def test_thousands_of_records_in_one_ring(mix):
+    """More failures than the host sets up claim words at a time, and none reused."""
+    name, c, d, p = mix[0]
+    s = synd_host(c, d, 0.2, 4000, 8200)
+    ref = alone(d, s)
+    assert (ref["stage"] != 0).sum() > 2100
+    srv = B.Server([d], max_inflight_shots=4096)
+    try:
+        tickets = [srv.submit(0, s[a:a + 500]) for a in range(0, 4000, 500)]
+        parts = [srv.poll(t, 500, 0) for t in tickets]
+        same({key: np.concatenate([g[key] for g in parts]) for key in ref}, ref)
+    finally:
+        srv.stop()
