@@ -178,8 +178,9 @@ static cudaError_t blocks_per_sm(const void *fn, int block, int smem, int *occ) 
 // rows of up to sixteen.  [[254]] at p = 0.04, column path against the best team
 // shape: 500 shots 0.18 / 0.48 ms, 5000 0.65 / 1.55, 50 000 5.6 / 10.3; at
 // p = 0.06 50 000 shots 21.4 / 43.0.  Blocks of 24 warps instead of 19 left 72
-// registers and spilled: [[254]] 5.57 -> 5.68 ms, 3000 [[288]] shots 0.57 -> 0.64
-// (only 20 000 [[72]] shots gained, 0.94 -> 0.86).
+// registers and spilled more than the 28 B a thread of the (10, 5) instance at 96:
+// [[254]] 5.57 -> 5.68 ms, 3000 [[288]] shots 0.57 -> 0.64 (only 20 000 [[72]]
+// shots gained, 0.94 -> 0.86).
 constexpr long long kColumnShots = 1500000;
 
 // Long codes (more than kMaxShardNnz edges; up to eight ones per row and three
@@ -187,10 +188,16 @@ constexpr long long kColumnShots = 1500000;
 // any batch.  In teams of four warps with a slot each, three warps waited while
 // one packed and installed 2592 columns.  10^5 shots of the 12-round
 // phenomenological [[144]] at p = q = 0.004: 7.6 ms in such teams, 4.6 with 27
-// warps on four slots, 4.7 with 19 warps, 5.7 with 27 on two slots.  Exact (6, 3)
-// codes have their own team loop, which wins where it does against the other
-// column path: 784 columns at p = 0.05, 1000 shots 1.01 against 0.97 ms, 20 000
-// 15.7 / 11.7; at p = 0.01 0.32 / 0.30 and 0.86 / 0.62.
+// warps on four slots, 4.7 with 19 warps, 5.7 with 27 on two slots.  150 calls of
+// other long codes (phenomenological, of 270 to 1008 rows at p = 0.002 to 0.01,
+// and irregular ones; 16 to 30 000 shots) read 1.29 times the speed of their
+// default teams in the geometric mean, from 0.77 to 2.75 times; below 1 at 30 000
+// runs of few iterations on 270 to 432 rows, and for some at 16 shots.  A code
+// whose four slots do not fit in a block (12 rounds of [[144]] take 172 KB, 18
+// rounds of it or 9 of [[288]] too much) stays on teams.  Exact (6, 3) codes have
+// their own team loop, which wins where it does against the other column path:
+// 784 columns at p = 0.05, 1000 shots 1.01 against 0.97 ms, 20 000 15.7 / 11.7; at
+// p = 0.01 0.32 / 0.30 and 0.86 / 0.62.
 static bool plan_long(bpsf_ctx *const *codes, int n_codes, const bpsf_tuning *tunes, const long long *shots, bool exact,
                       bpsf_plan *out, int *variant, int *B, int *smem, int Q) {
     int bytes = 0;

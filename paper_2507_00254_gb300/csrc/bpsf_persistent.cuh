@@ -910,8 +910,8 @@ __device__ void team_loop(const StreamDev &sd, const LayoutMem &L, const TeamMem
     // Layered schedule: vector lanes in the full-register instances only.
     constexpr bool kLayV2 = LAY && kVec && MINB == 1 && DC <= 6, kLayV4 = kLayV2 && kVec4;
     const bool lay = LAY && cd.layered;
-    // The 64-register instance has no registers for this: it spilled, and 200 000
-    // [[72]] shots took 6.6 instead of 5.7 ms.
+    // Not in the 64-register instance: it spills 32 B a thread as it is, and with
+    // this 200 000 [[72]] shots took 6.6 instead of 5.7 ms.
     Hot h = {cd.M, cd.N, cd.Mp, cd.vchk, false, 0.f};
     if (MINB == 1) h = {keep(h.M), keep(h.N), keep(h.Mp), keep(h.vchk), keep(cd.uniform) != 0 && !lay, cd.lch0};
     const float alpha0 = cd.alpha;
